@@ -11,6 +11,22 @@ constexpr int kMaxN3D = 6;      // 3D builds degree <= 5
 constexpr int kMaxRing = 24;    // ring levels (random_delay_max + np + 1 <= 15 + 7 + 1)
 constexpr int kMaxCoefDelay = 16;
 
+// Fixed-point operator tables of the FP64 contractions (fixline.cuh).  eout: exponent of a
+// result relative to that of its values; elo, ehi: value exponents the tables cover.
+struct FixedScale {
+  int eout, elo, ehi;
+};
+struct FixedTrace {  // rows l_a(-1) and l_a(+1), the limbs of an entry side by side
+  int2 t[2][kMaxN];
+  long long c[2];  // start values of the middle limb sums (fixline.cuh)
+  FixedScale s;
+};
+struct FixedSweep {  // direction d, row i: N flux weights, low-face and high-face weight
+  int2 q[3][kMaxN * (kMaxN + 2)];  // entry [i*(N+2) + k]
+  long long c[3][kMaxN];           // start value of the middle limb sum per row (fixline.cuh)
+  FixedScale s;                    // one scale for all directions
+};
+
 // Operator tables in FP64; kernels convert entries to their arithmetic type.
 struct OpTables {
   double Q[3][kMaxN * kMaxN];  // (2/h_d) omega_a l_i'(xi_a) / omega_i, entry [i*N + a]
@@ -37,25 +53,33 @@ struct OpTables {
   float2 Qsf[3][kMaxN * kMaxN];
   float2 Lpsf[3][kMaxN];
   float2 Lmsf[3][kMaxN];
+  // the tables (unscaled and dt-scaled) and the trace weights in fixed point
+  FixedSweep fx, fxs;
+  FixedTrace ft;
 };
 
 struct MeshArgs {
   int n[3];
   int64_t ne;
   int64_t es[3];  // element index stride per direction
-  // Division by n[0] and n[1] as a multiply-high (division by invariant integers, Granlund
-  // & Montgomery, PLDI 1994): q = floor(e / n) = umulhi64(e, M) with M = ceil(2^64 / n),
-  // exact for e < 2^64 / n, hence for every 32-bit e when n < 2^31; n = 1 is special-cased.
-  uint64_t divm[2];
+  // Division by n[0] and n[1] as a 32-bit multiply-high and a shift (division by invariant
+  // integers, Granlund & Montgomery, PLDI 1994): with 2^(l-1) < n <= 2^l and
+  // M = floor(2^(31+l) / n) + 1 < 2^32, floor(e / n) = (e M) >> (31 + l) for 0 <= e < 2^31
+  // (e (M n - 2^(31+l)) <= e 2^l < 2^(31+l)); n = 1 is special-cased.
+  uint32_t divm[2], divs[2];
 };
 
-// Fills es[] and divm[] from n[] (host side).
+// Fills es[], divm[] and divs[] from n[] (host side), n[0], n[1] <= 2^20.
 inline void mesh_finish(MeshArgs& m) {
   m.es[0] = 1;
   m.es[1] = m.n[0];
   m.es[2] = (int64_t)m.n[0] * m.n[1];
-  for (int i = 0; i < 2; ++i)
-    m.divm[i] = m.n[i] > 1 ? ~0ull / (uint64_t)m.n[i] + 1ull : 0ull;
+  for (int i = 0; i < 2; ++i) {
+    uint32_t l = 0;
+    while (((uint32_t)1 << l) < (uint32_t)m.n[i]) ++l;
+    m.divm[i] = l > 0 ? (uint32_t)(((uint64_t)1 << (31 + l)) / (uint64_t)m.n[i] + 1) : 0;
+    m.divs[i] = l > 0 ? l - 1 : 0;
+  }
 }
 
 enum UpdateMode { kModeRHS = 0, kMode2R = 1, kMode2N = 2 };
@@ -83,6 +107,7 @@ struct __align__(16) VolArgs {
   int scaled;            // 1: use the dt-scaled tables (2N), the accumulator is dt * k
   int bulk;              // 1: n_elem * nodes is a multiple of 4, so the element path may
                          // stage whole tiles by TMA bulk copies (16-byte aligned rows)
+  FixedTrace ft;         // trace weights (FP64 trace arithmetic)
 };
 
 struct __align__(16) FluxArgs {
@@ -129,6 +154,7 @@ struct TraceArgs {
   const OpTables* tab;
   const double* u;
   void* tr;
+  FixedTrace ft;  // trace weights (FP64 trace arithmetic)
 };
 
 // Learned correction of subdomain traces (learned.cu).

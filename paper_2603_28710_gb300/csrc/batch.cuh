@@ -96,6 +96,27 @@ batch_vol_kernel(const VolArgs* va, int nstages, int stage, BatchGroupArgs g) {
   }
 }
 
+template <int D, int N, int TT>
+__global__ void __launch_bounds__(VolSmem64<D, N, TT>::BLOCK,
+                                  min_blocks_for(VolRegs<D, N, double>::value, VolSmem64<D, N, TT>::BLOCK))
+batch_vol_kernel_fp64(const VolArgs* va, int nstages, int stage, BatchGroupArgs g) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) VolArgs sa;
+  __shared__ int soff[kMaxSharedOffsets];
+  const int* off = stage_offsets(g, soff);
+  int cur = -1;  // instance whose arguments sa holds (uniform over the block)
+  for (int vb = blockIdx.x; vb < g.total; vb += gridDim.x) {
+    const int k = find_instance(off, g.n, vb);
+    if (k != cur) {
+      stage_args(&sa, &va[g.inst[k] * nstages + stage]);
+      __syncthreads();
+      cur = k;
+    }
+    vol_body_fp64<D, N, TT>(sa, vb - off[k], smem_raw);
+    __syncthreads();  // shared memory (and the arguments) are reused by the next virtual block
+  }
+}
+
 // Element path of the batch (FP32 operator): the volume kernel with every element
 // evaluating the numerical fluxes on its own faces, reading each instance's stage and face
 // arguments (the face arguments carry the schedule the device advances) from shared
@@ -159,16 +180,21 @@ struct BatchDispatch {
   static cudaError_t vol_t(const VolArgs* va, int ns, int st, const BatchGroupArgs& g, int grid,
                            cudaStream_t s, int* occ) {
     using T = Tile<D, N, TT>;
-    const size_t smem = vol_flux_bytes<D, N, R, TT>();
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(batch_vol_kernel<D, N, R, TT>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
+    if constexpr (std::is_same<R, double>::value) {
+      return go(batch_vol_kernel_fp64<D, N, TT>, VolSmem64<D, N, TT>::BLOCK, VolSmem64<D, N, TT>::BYTES, va, ns,
+                st, g, grid, s, occ);
+    } else {
+      return go(batch_vol_kernel<D, N, R, TT>, T::THREADS, vol_flux_bytes<D, N, R, TT>(), va, ns, st, g,
+                grid, s, occ);
     }
-    if (occ)
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_vol_kernel<D, N, R, TT>,
-                                                           T::THREADS, smem);
-    batch_vol_kernel<D, N, R, TT><<<grid, T::THREADS, smem, s>>>(va, ns, st, g);
+  }
+  template <typename K>
+  static cudaError_t go(K kernel, int threads, size_t smem, const VolArgs* va, int ns, int st,
+                        const BatchGroupArgs& g, int grid, cudaStream_t s, int* occ) {
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
+    if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, threads, smem);
+    kernel<<<grid, threads, smem, s>>>(va, ns, st, g);
     return cudaGetLastError();
   }
   template <int D, int N, int TT>

@@ -107,7 +107,9 @@ struct FusedSmem {
   static constexpr size_t BIG = 2 * SLOT;
   static constexpr size_t FF = BIG + BIGB;
   static constexpr size_t BAR = FF + FFB;
-  static constexpr size_t BYTES = BAR + 16;
+  static constexpr size_t MAXOFF = BAR + 16;  // largest magnitudes per element and variable (FP64)
+  static constexpr size_t BYTES =
+      MAXOFF + (std::is_same<R, double>::value ? sizeof(int) * F::EPB * F::NV : 0);
 };
 
 // ---- TMA tensor copies (PTX; the mbarrier helpers are in kernels.cuh) -------------
@@ -176,6 +178,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
   R* sFF = reinterpret_cast<R*>(smem + SM::FF);
   float2* sFF2 = reinterpret_cast<float2*>(smem + SM::FF);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + SM::BAR);
+  int* sMax = reinterpret_cast<int*>(smem + SM::MAXOFF);
 
   const VolArgs& V = A.v;
   const MeshArgs& m = V.m;
@@ -288,7 +291,21 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
     __syncthreads();
 
     // ---- B1. traces of the tile's elements on all their faces (from U) -------------------
-    {
+    if constexpr (std::is_same<R, double>::value) {
+      constexpr int CT = D * NV * NF;  // (direction, variable, line) combinations
+      for (int g = tid; g < CT * EPB; g += THREADS) {
+        const int c = g % CT, te = g / CT;
+        const int j = c % NF, dv = c / NF;
+        const int v = dv % NV, d = dv / NV;
+        const double* x = sUin + v * ROW + te * ND + line_base<D, N>(d, j);
+        const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+        double val[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) val[a] = x[a * stride];
+        double* t = sT + ((te * 2 * D + 2 * d) * NV + v) * NF + j;
+        line_traces<N>(V.ft, V.tab, val, t[0], t[NV * NF]);
+      }
+    } else {
       constexpr int CT = 2 * D * NV * NF;  // (direction, side, variable, face node) combinations
       for (int g = tid; g < CT * EPB; g += THREADS) {
         const int c = g % CT, te = g / CT;
@@ -374,6 +391,19 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
     __syncthreads();
 
     // ---- B2. pointwise Euler fluxes (over U and T, both no longer needed) -----------------
+    // face ds = 2 d + side of this thread's element: low plane = its own tile coordinate
+    auto face_of = [=](int ds) {
+      const int d = ds >> 1;
+      const int lo = d == 0 ? (ez * TY + ey) * (TX + 1) + ex
+                            : (d == 1 ? F::F0 + (ez * (TY + 1) + ey) * TX + ex
+                                      : F::F0 + F::F1 + (ez * TY + ey) * TX + ex);
+      return (ds & 1) ? lo + (d == 0 ? 1 : (d == 1 ? TX : TX * TY)) : lo;
+    };
+    // FP64: sweep tables, exponents per variable, FP64 chain needed
+    const FixedSweep* ftab = V.scaled ? &V.tab->fxs : &V.tab->fx;
+    const FixedScale fsc = ftab->s;
+    int fex[NV];
+    bool chain = false;
     {
       R Fp[D][NV];
       euler_flux_all<D, R>(u, Arith<R>::pair(V.gm1, V.gm1f), Fp);
@@ -384,6 +414,37 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           for (int pr = 0; pr < NP; ++pr)
             sF2[((el * D + d) * NP + pr) * ND + node] =
                 make_float2(Fp[d][2 * pr], 2 * pr + 1 < NV ? Fp[d][2 * pr + 1] : 0.0f);
+      } else if constexpr (std::is_same<R, double>::value) {
+        // fixed point as in vol_body_fp64: per element and variable one exponent over the
+        // pointwise fluxes and the fluxes on the element's faces
+        for (int i = tid; i < EPB * NV; i += THREADS) sMax[i] = 0;
+        __syncthreads();
+        if (active) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            int mx = abs_hi(Fp[0][v]);
+#pragma unroll
+            for (int d = 1; d < D; ++d) mx = max(mx, abs_hi(Fp[d][v]));
+            for (int q = node; q < 2 * D * NF; q += ND) {
+              const int ds = q / NF, j = q - ds * NF;
+              mx = max(mx, abs_hi(sFF[(face_of(ds) * NV + v) * NF + j]));
+            }
+            atomicMax(sMax + el * NV + v, mx);
+          }
+        }
+        __syncthreads();
+        if (active) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            fex[v] = fixed_exponent(fsc, sMax[el * NV + v]);
+            chain = chain || fex[v] > fsc.ehi;
+          }
+#pragma unroll
+          for (int d = 0; d < D; ++d)
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+              sF[((el * D + d) * NV + v) * ND + node] = chain ? Fp[d][v] : fixed_bits(Fp[d][v], fex[v] + kSweepShift);
+        }
       } else {
 #pragma unroll
         for (int d = 0; d < D; ++d)
@@ -399,14 +460,47 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] = acc_zero(Acc());
     if (active) {
-      // faces of this element along d: low plane = its own tile coordinate, high = +1
-      int flo[3], fhi[3];
-      flo[0] = (ez * TY + ey) * (TX + 1) + ex;
-      fhi[0] = flo[0] + 1;
-      flo[1] = F::F0 + (ez * (TY + 1) + ey) * TX + ex;
-      fhi[1] = flo[1] + TX;
-      flo[2] = F::F0 + F::F1 + (ez * TY + ey) * TX + ex;
-      fhi[2] = flo[2] + TX * TY;
+      int flo[3], fhi[3];  // faces of this element along d
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        flo[d] = face_of(2 * d);
+        fhi[d] = face_of(2 * d + 1);
+      }
+      bool fixed = false;
+      if constexpr (std::is_same<R, double>::value) {
+        if (!chain) {
+          fixed = true;
+          FixedAcc fa[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            fa[v] = FixedAcc{0, 0};
+#pragma unroll
+            for (int d = 0; d < D; ++d) fa[v].m += ftab->c[d][ix[d]];
+          }
+#pragma unroll
+          for (int d = 0; d < D; ++d) {
+            const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+            const int base = node - ix[d] * stride, j = face_index<D, N>(d, ix);
+            const int2* q = ftab->q[d] + ix[d] * (N + 2);
+#pragma unroll
+            for (int a = 0; a < N; ++a)
+#pragma unroll
+              for (int v = 0; v < NV; ++v)
+                fixed_fma(q[a], fixed_of_bits(sF[((el * D + d) * NV + v) * ND + base + a * stride]), fa[v]);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+              int2 flw = fixed_limbs(sFF[(flo[d] * NV + v) * NF + j], fex[v] + kSweepShift);
+              int2 fhw = fixed_limbs(sFF[(fhi[d] * NV + v) * NF + j], fex[v] + kSweepShift);
+              opaque(flw);
+              opaque(fhw);
+              fixed_fma(q[N], flw, fa[v]);
+              fixed_fma(q[N + 1], fhw, fa[v]);
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc[v] = fixed_result(fa[v], fsc, fex[v]);
+        }
+      }
       if constexpr (PK) {
         float2 a2[NP];
 #pragma unroll
@@ -441,7 +535,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
 #pragma unroll
           for (int v = 0; v < NV; ++v) acc[v] = (v & 1) ? a2[v / 2].y : a2[v / 2].x;
         }
-      } else {
+      } else if (!fixed) {
 #pragma unroll
         for (int d = 0; d < D; ++d) {
           const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
@@ -545,14 +639,23 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           x = a0; y = a1; z = side ? E2 - 1 : 0;
         }
         const int te = (z * TY + y) * TX + x;
-        const int base = line_base<D, N>(d, j);
+        const C* src = sN + v * ROW + te * ND + line_base<D, N>(d, j);
         const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
-        const double* tw = side ? V.tab->Tp : V.tab->Tm;
-        const float2* twf = side ? V.tab->Tpf : V.tab->Tmf;
-        C t[N];
+        C val;
+        if constexpr (std::is_same<R, double>::value) {
+          double line[N], lo, hi;
 #pragma unroll
-        for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
-        const C val = interp_line<N, C>(t, sN + v * ROW + te * ND + base, stride);
+          for (int a = 0; a < N; ++a) line[a] = src[a * stride];
+          line_traces<N>(V.ft, V.tab, line, lo, hi);
+          val = side ? hi : lo;
+        } else {
+          const double* tw = side ? V.tab->Tp : V.tab->Tm;
+          const float2* twf = side ? V.tab->Tpf : V.tab->Tmf;
+          C t[N];
+#pragma unroll
+          for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
+          val = interp_line<N, C>(t, src, stride);
+        }
         store_trace(tro + (((d * 2 + side) * NV + v) * ne + gel(x, y, z)) * NF + j, val);
       }
     }

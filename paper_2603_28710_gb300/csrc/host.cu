@@ -2,6 +2,7 @@
 // delay schedules and the per-stage launch sequence.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -113,6 +114,83 @@ void lagrange_at(int n, const long double* x, const long double* lam, long doubl
   for (int j = 0; j < n; ++j) out[j] = (lam[j] / (y - x[j])) / den;
 }
 
+// ---- fixed-point tables of the FP64 contractions (fixline.cuh) ------------------------
+constexpr int kFixedSumBits = 61;  // bound of a contraction's sum of |entries|, in bits
+
+// limbs of a fixed-point table entry: v = x 2^31 + y, |y| <= 2^30
+int2 fixed_entry(int64_t v) {
+  const int64_t hi = (v + ((int64_t)1 << 30)) >> 31;
+  return make_int2((int)hi, (int)(v - hi * ((int64_t)1 << 31)));
+}
+
+// Exponents for a table stored as value 2^sq whose 64-bit results are value 2^-eout of the
+// values' exponent: results have to be normal numbers.
+FixedScale fixed_scale(int eout) {
+  FixedScale f;
+  f.eout = eout;
+  f.elo = eout < 4 ? 64 - eout : 60;
+  f.ehi = eout > -1 ? 2045 - eout : 2046;
+  return f;
+}
+
+// largest row sum of |v| of a rows x cols table
+template <typename T>
+T row_sum_max(const T* v, int rows, int cols) {
+  T big = 0;
+  for (int i = 0; i < rows; ++i) {
+    T sum = 0;
+    for (int k = 0; k < cols; ++k) sum += v[i * cols + k] < 0 ? -v[i * cols + k] : v[i * cols + k];
+    big = sum > big ? sum : big;
+  }
+  return big;
+}
+
+// power of two that brings a sum of |entries| to at most 2^kFixedSumBits
+int fixed_shift(long double sum) {
+  int ex = 0;
+  frexpl(sum, &ex);  // sum < 2^ex
+  return kFixedSumBits - ex;
+}
+
+// Sweep tables times dt (scaled) or as they are, from the integers of build_tables: an integer
+// product with the mantissa of dt.  One scale for all directions, whose sum a contraction
+// forms; entries are halved once more where the middle limb sum of the worst row,
+// sum |q1| 2^31 + |q0| 2^28, could reach 2^63.
+void fixed_sweep_tables(const adg_solver* s, double dt, bool scaled, FixedSweep* f) {
+  const int N = s->N, M = N + 2;
+  int ex = 0;
+  const int64_t mant = scaled ? (int64_t)std::ldexp(std::frexp(dt, &ex), 53) : 0;  // dt = mant 2^(ex-53)
+  int sh = 0;
+  if (scaled) {
+    __int128 sum = 0;
+    for (int d = 0; d < s->dim; ++d) sum += (__int128)row_sum_max(s->fix_q[d], N, M) * mant;
+    sh = (sum >> 52) <= ((__int128)1 << kFixedSumBits) ? 52 : 53;
+  }
+  for (;; ++sh) {
+    unsigned __int128 worst = 0;
+    for (int d = 0; d < s->dim; ++d) {
+      unsigned __int128 big = 0;
+      for (int i = 0; i < N; ++i) {
+        unsigned __int128 sum = 0;
+        f->c[d][i] = d == 0 ? (long long)1 << 30 : 0;
+        for (int k = 0; k < M; ++k) {
+          const __int128 v = (__int128)s->fix_q[d][i * M + k] * (scaled ? mant : 1);
+          const int2 q = fixed_entry((int64_t)(sh > 0 ? (v + ((__int128)1 << (sh - 1))) >> sh : v));
+          f->q[d][i * M + k] = q;
+          f->c[d][i] += q.y / 2;
+          sum += ((unsigned __int128)(q.x < 0 ? -(int64_t)q.x : q.x) << 31) +
+                 ((unsigned __int128)(q.y < 0 ? -(int64_t)q.y : q.y) << 28);
+        }
+        big = sum > big ? sum : big;
+      }
+      worst += big;
+    }
+    if (worst >> 63 == 0) break;
+  }
+  // value 2^sq with sq = fix_s + 53 - sh - ex (scaled) or fix_s - sh
+  f->s = fixed_scale(67 - (scaled ? s->fix_s + 53 - sh - ex : s->fix_s - sh));
+}
+
 void build_tables(adg_solver* s) {
   const int N = s->N;
   OpTables& T = s->tab;
@@ -163,6 +241,35 @@ void build_tables(adg_solver* s) {
     T.Tm[a] = (double)lm[a];
     T.Tpf[a] = split2(lp[a]);
     T.Tmf[a] = split2(lm[a]);
+  }
+  // the same rows in fixed point: per direction N flux weights, low and high face
+  {
+    const int M = N + 2;
+    long double rows[3][kMaxN * (kMaxN + 2)], sum = 0.0L;
+    for (int d = 0; d < s->dim; ++d) {
+      const long double sc = 2.0L / (long double)s->h[d];
+      for (int i = 0; i < N; ++i) {
+        for (int a = 0; a < N; ++a)
+          rows[d][i * M + a] = sc * (long double)wd[a] * Dm[a][i] / (long double)wd[i];
+        rows[d][i * M + N] = 0.5L * sc * lm[i] / (long double)wd[i];
+        rows[d][i * M + N + 1] = -0.5L * sc * lp[i] / (long double)wd[i];
+      }
+      sum += row_sum_max(rows[d], N, M);
+    }
+    s->fix_s = fixed_shift(sum);
+    for (int d = 0; d < s->dim; ++d)
+      for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[d][i], s->fix_s));
+    fixed_sweep_tables(s, 0.0, false, &T.fx);
+    const int st = fixed_shift(std::max(row_sum_max(lm, 1, N), row_sum_max(lp, 1, N)));
+    for (int a = 0; a < N; ++a) {
+      T.ft.t[0][a] = fixed_entry((int64_t)llroundl(ldexpl(lm[a], st)));
+      T.ft.t[1][a] = fixed_entry((int64_t)llroundl(ldexpl(lp[a], st)));
+    }
+    for (int side = 0; side < 2; ++side) {
+      T.ft.c[side] = (long long)1 << 30;
+      for (int a = 0; a < N; ++a) T.ft.c[side] += T.ft.t[side][a].y / 2;
+    }
+    T.ft.s = fixed_scale(66 - st);
   }
   double xe[16], we[16];
   gauss_legendre(N + 1, xe, we);
@@ -428,6 +535,7 @@ adg_status launch_traces_of(adg_solver* s, const double* u) {
   ta.tab = s->tab_dev;
   ta.u = u;
   ta.tr = s->tr;
+  ta.ft = s->tab.ft;
   ADG_CUDA(s, launch_trace(s->prec, s->dim, s->N, ta, s->stream));
   return ADG_OK;
 }
@@ -503,6 +611,7 @@ adg_status upload_dt_tables(adg_solver* s) {
       s->tab.Lmsf[d][i] = split2((long double)s->tab.Lm[d][i] * s->dt);
     }
   }
+  fixed_sweep_tables(s, s->dt, true, &s->tab.fxs);
   ADG_CUDA(s, cudaMemcpyAsync(s->tab_dev, &s->tab, sizeof(OpTables), cudaMemcpyHostToDevice, s->stream));
   return ADG_OK;
 }
@@ -623,13 +732,15 @@ VolArgs stage_vol_args(const adg_solver* s, int m) {
   va.write_traces = 1;
   va.scaled = s->rk2n ? 1 : 0;
   va.bulk = (s->ne * s->ND) % 4 == 0 ? 1 : 0;
+  va.ft = s->tab.ft;
   return va;
 }
 
 // Helpers for adg_rhs_noalloc (noalloc.cu): the same operator tables without a handle,
 // and the per-thread error text that adg_last_error(NULL) returns.
-void noalloc_build_tables(int N, const double* h, OpTables* T) {
+void noalloc_build_tables(int dim, int N, const double* h, OpTables* T) {
   adg_solver tmp;
+  tmp.dim = dim;
   tmp.N = N;
   for (int d = 0; d < 3; ++d) tmp.h[d] = h[d];
   build_tables(&tmp);

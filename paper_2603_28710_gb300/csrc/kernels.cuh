@@ -7,7 +7,7 @@
 //   flux_kernel : one thread per (direction, face, face node): numerical flux of Eq. 8-9
 //                 from the two stored traces; on faces between subdomains it applies the
 //                 delayed / AT rules of Algorithms 2-3 (Eq. 13-14) against a ring buffer.
-//   vol_kernel  : one thread per node, a tile of elements per block: pointwise Euler flux
+//   vol_kernel (FP64: vol_kernel_fp64) : one thread per node, a tile of elements per block: pointwise Euler flux
 //                 (Eq. 2), sum-factorised weak derivative along each direction, face lift,
 //                 inverse mass (diagonal for collocated Gauss points; folded into the
 //                 tables), the low-storage RK update (Eq. 10 or the 2N form), and the
@@ -23,6 +23,7 @@
 
 #include "adg_internal.h"
 #include "arith.cuh"
+#include "fixline.cuh"
 
 namespace adg {
 
@@ -62,7 +63,7 @@ constexpr int sx_stride() {  // next stage input [el][NV][ND]
 
 // floor(e / m.n[i]) for 0 <= e < 2^31 (multiply-high by the precomputed inverse)
 __device__ __forceinline__ int mesh_div(const MeshArgs& m, int i, int e) {
-  return m.n[i] == 1 ? e : (int)__umul64hi((unsigned long long)(unsigned)e, m.divm[i]);
+  return m.n[i] == 1 ? e : (int)(__umulhi((unsigned)e, m.divm[i]) >> m.divs[i]);
 }
 
 // Blocks per SM that leave `regs` registers per thread (0: no budget): each of the 4 SM
@@ -277,65 +278,81 @@ __device__ __forceinline__ void store_trace(float2* p, double v) {
 }
 __device__ __forceinline__ void store_trace(float2* p, df64 v) { *p = make_float2(v.hi, v.lo); }
 
-// Traces of a tile of elements held in shared memory sX[el][v][node] (compute type C,
-// element stride SXS) -> tr.
-// FP32 and FP32-pair operators: a thread owns one (direction, side, variable, face node)
-// combination, so its line of nodes, stride and interpolation weights are set up once, and
-// interpolates it for a run of the tile's elements (the runs split the elements when the
-// block has threads to spare); this halves their instruction count in this phase.  The
-// FP64 operator is bound by its FP64 pipe, not by issue, and keeps one flat loop over all
-// (element, face node) items, which spreads the FP64 work over every thread.
-template <int D, int N, typename R, int TT = 128, typename C = R,
-          int SXS = (D + 2) * IPow<N, D>::value>
+// FP64 traces of a tile of elements in shared memory (value (el, v, node) at v * VS + el * ND +
+// node) -> tr: one thread per (direction, variable, line) interpolates both ends of
+// its line in fixed point (fixline.cuh).
+template <int D, int N, int TT>
+__device__ __forceinline__ void write_traces_fp64(const MeshArgs& m, const FixedTrace& ft,
+                                                  const OpTables* tab, const double* sX, int VS,
+                                                  int e0, double* tr) {
+  using T = Tile<D, N, TT>;
+  constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB, LINES = EPB * NF;
+  const int ne = (int)m.ne;
+  const int last = (ne - e0) * NF;  // lines of the tile's elements inside the mesh
+  for (int g = threadIdx.x; g < D * NV * LINES; g += blockDim.x) {
+    const int dv = g / LINES, r = g - dv * LINES;  // r = el * NF + j
+    const int d = dv / NV, v = dv - d * NV;
+    if (r >= last) continue;
+    const double* x = sX + v * VS;
+    int st = 1;
+    if (d == 0) {
+      x += r * N;  // line j of an element starts at its node j * N
+    } else {
+      const int el = r / NF;
+      x += r + el * (ND - NF);
+      st = N;
+      if constexpr (D == 3) {
+        if (d == 1) x += (r - el * NF) / N * (N * N - N);
+        else st = N * N;
+      }
+    }
+    double val[N], lo, hi;
+#pragma unroll
+    for (int a = 0; a < N; ++a) val[a] = x[a * st];
+    line_traces<N>(ft, tab, val, lo, hi);
+    double* dst = tr + ((2 * d * NV + v) * ne + e0) * NF + r;
+    dst[0] = lo;
+    dst[NV * ne * NF] = hi;
+  }
+}
+
+// Traces of a tile of elements held in shared memory sX[el][v][node] (compute type C, element
+// stride SXS) -> tr, FP32 and FP32-pair operators: a thread owns one (direction, side,
+// variable, face node) combination, so its line of nodes, stride and interpolation weights
+// are set up once, and interpolates it for a run of the tile's elements (the runs split the
+// elements when the block has threads to spare); this halves the instruction count of this
+// phase.  (The pair kernels are bound by issue as much as by the FP64 pipe: fixed-point lines
+// as in the FP64 operator cost them 15 %.)
+template <int D, int N, typename R, int TT, typename C, int SXS>
 __device__ __forceinline__ void write_traces(const MeshArgs& m, const OpTables* tab, const C* sX,
                                              int e0, typename Arith<R>::S* tr) {
   using T = Tile<D, N, TT>;
   constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB;
   const int ne = (int)m.ne;
-  if constexpr (std::is_same<R, double>::value) {
-    constexpr int TOTAL = EPB * 2 * D * NV * NF;
-    for (int g = threadIdx.x; g < TOTAL; g += blockDim.x) {
-      const int jj = g % (EPB * NF);
-      const int rest = g / (EPB * NF);  // (d*2 + side)*NV + v
-      const int el = jj / NF, j = jj - el * NF;
-      const int e = e0 + el;
-      if (e >= ne) continue;
-      const int v = rest % NV, ds = rest / NV;
-      const int d = ds >> 1, side = ds & 1;
-      const int base = line_base<D, N>(d, j);
-      const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
-      const double* tw = side ? tab->Tp : tab->Tm;
-      double acc = 0.0;
+  constexpr int CT = 2 * D * NV * NF;                            // combinations
+  constexpr int CH = T::THREADS / CT > 0 ? T::THREADS / CT : 1;  // element runs
+  constexpr int RUN = (EPB + CH - 1) / CH;                       // elements per run
+  for (int g = threadIdx.x; g < CT * CH; g += blockDim.x) {
+    const int c = g % CT, ch = g / CT;
+    const int j = c % NF, rest = c / NF;  // rest = (d*2 + side)*NV + v
+    const int v = rest % NV, ds = rest / NV;
+    const int d = ds >> 1, side = ds & 1;
+    const int base = line_base<D, N>(d, j);
+    const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+    const double* tw = side ? tab->Tp : tab->Tm;
+    const float2* twf = side ? tab->Tpf : tab->Tmf;
+    C t[N];
 #pragma unroll
-      for (int a = 0; a < N; ++a) acc = fma(tw[a], sX[el * SXS + v * ND + base + a * stride], acc);
-      store_trace(tr + ((ds * NV + v) * ne + e) * NF + j, acc);
-    }
-  } else {
-    constexpr int CT = 2 * D * NV * NF;                            // combinations
-    constexpr int CH = T::THREADS / CT > 0 ? T::THREADS / CT : 1;  // element runs
-    constexpr int RUN = (EPB + CH - 1) / CH;                       // elements per run
-    for (int g = threadIdx.x; g < CT * CH; g += blockDim.x) {
-      const int c = g % CT, ch = g / CT;
-      const int j = c % NF, rest = c / NF;  // rest = (d*2 + side)*NV + v
-      const int v = rest % NV, ds = rest / NV;
-      const int d = ds >> 1, side = ds & 1;
-      const int base = line_base<D, N>(d, j);
-      const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
-      const double* tw = side ? tab->Tp : tab->Tm;
-      const float2* twf = side ? tab->Tpf : tab->Tmf;
-      C t[N];
+    for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
+    const int el0 = ch * RUN;
+    const int el1 = el0 + RUN < EPB ? el0 + RUN : EPB;
+    typename Arith<R>::S* dst = tr + ((ds * NV + v) * ne + e0) * NF + j;
+    for (int el = el0; el < el1 && e0 + el < ne; ++el) {
+      const C* x = sX + el * SXS + v * ND + base;
+      typename Arith<C>::Acc acc = acc_zero(typename Arith<C>::Acc());
 #pragma unroll
-      for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
-      const int el0 = ch * RUN;
-      const int el1 = el0 + RUN < EPB ? el0 + RUN : EPB;
-      typename Arith<R>::S* dst = tr + ((ds * NV + v) * ne + e0) * NF + j;
-      for (int el = el0; el < el1 && e0 + el < ne; ++el) {
-        const C* x = sX + el * SXS + v * ND + base;
-        typename Arith<C>::Acc acc = acc_zero(typename Arith<C>::Acc());
-#pragma unroll
-        for (int a = 0; a < N; ++a) acc = acc_fma(t[a], x[a * stride], acc);
-        store_trace(dst + el * NF, acc_result(acc));
-      }
+      for (int a = 0; a < N; ++a) acc = acc_fma(t[a], x[a * stride], acc);
+      store_trace(dst + el * NF, acc_result(acc));
     }
   }
 }
@@ -354,10 +371,15 @@ __global__ void __launch_bounds__(Tile<D, N>::THREADS) trace_kernel(const TraceA
   if (e < ne) {
 #pragma unroll
     for (int v = 0; v < NV; ++v)
-      sX[(el * NV + v) * ND + node] = Arith<C>::from_double(A.u[(v * ne + e) * ND + node]);
+      sX[std::is_same<R, double>::value ? v * T::THREADS + (int)threadIdx.x : (el * NV + v) * ND + node] =
+          Arith<C>::from_double(A.u[(v * ne + e) * ND + node]);
   }
   __syncthreads();
-  write_traces<D, N, R, 128, C>(A.m, A.tab, sX, e0, reinterpret_cast<typename Arith<R>::S*>(A.tr));
+  typename Arith<R>::S* tr = reinterpret_cast<typename Arith<R>::S*>(A.tr);
+  if constexpr (std::is_same<R, double>::value)
+    write_traces_fp64<D, N, 128>(A.m, A.ft, A.tab, sX, T::THREADS, e0, tr);
+  else
+    write_traces<D, N, R, 128, C, NV * ND>(A.m, A.tab, sX, e0, tr);
 }
 
 // ---- Runge-Kutta update of one node -------------------------------------------------
@@ -423,17 +445,15 @@ struct Update {
   }
 };
 
+// FP64: w0 is the solution and q the 2N register at this index.
 template <>
 struct Update<double> {
-  __device__ static __forceinline__ double apply(const VolArgs& A, int idx, double k, double u_in,
-                                                 double& xd, bool = false, double = 0.0,
-                                                 double = 0.0) {
-    xd = 0.0;
+  __device__ static __forceinline__ double apply(const VolArgs& A, int idx, double k, double w0,
+                                                 double q) {
     if (A.mode == kModeRHS) {
       A.kout[idx] = k;
-      return u_in;
+      return k;
     }
-    const double w0 = A.w[idx];
     double* x = reinterpret_cast<double*>(A.x);
     if (A.mode == kMode2R) {
       const double w1 = fma(A.cb, k, w0);
@@ -443,8 +463,8 @@ struct Update<double> {
       x[idx] = r1;
       return r1;
     }
-    const double dtk = A.scaled ? k : A.dt * k;
-    const double q1 = A.stage > 0 ? fma(A.ca, x[idx], dtk) : dtk;
+    // (the 2N scheme takes the dt-scaled tables: k is dt times the right-hand side)
+    const double q1 = A.stage > 0 ? fma(A.ca, q, k) : k;
     const double w1 = fma(A.cb, q1, w0);
     A.w[idx] = w1;
     if (!A.last) x[idx] = q1;
@@ -503,8 +523,8 @@ struct ElementFaces {
 // The FP32 and FP32-pair forms wait on memory more than on their pipes: they stage their
 // stage input, solution and 2N register through shared memory with asynchronous copies
 // issued at the start, so the reads of the RK update are in flight during the volume work
-// instead of after it (512^2 p=4: FP32 210 -> 187 us, pairs 8 % faster).  The FP64 form is
-// bound by its FP64 pipe and keeps plain loads.
+// instead of after it (512^2 p=4: FP32 210 -> 187 us, pairs 8 % faster).  (FP64:
+// vol_body_fp64.)
 template <typename R> struct VolStages { static constexpr bool value = false; };
 template <> struct VolStages<float> { static constexpr bool value = true; };
 template <> struct VolStages<df64> { static constexpr bool value = true; };
@@ -769,6 +789,280 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned ch
   }
 }
 
+// ---- FP64 volume/update work --------------------------------------------------------
+
+// Elements that a warp of a tile of THREADS nodes touches, at most.
+template <int ND, int THREADS>
+constexpr int warp_elements() {
+  int most = 1;
+  for (int w = 0; w < THREADS; w += 32) {
+    const int end = (w + 31 < THREADS ? w + 31 : THREADS - 1) / ND - w / ND + 1;
+    most = end > most ? end : most;
+  }
+  return most;
+}
+
+// Maximum of m over the lanes of each element (el: this lane's element, -1: none) into
+// smax[el * NV + v]; lanes of one element are neighbours.
+template <int ND, int NV, int THREADS>
+__device__ __forceinline__ void element_max(const int (&m)[NV], int el, int* smax) {
+  if constexpr (ND < 16) {
+    if (el >= 0) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) atomicMax(smax + el * NV + v, m[v]);
+    }
+  } else {
+    // one warp reduction per element the warp touches, then one atomic per variable
+    const int lane = threadIdx.x & 31, first = (int)(threadIdx.x - lane) / ND;
+#pragma unroll
+    for (int k = 0; k < warp_elements<ND, THREADS>(); ++k) {
+      const bool in = el == first + k;
+      int mine = 0;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const int r = __reduce_max_sync(0xFFFFFFFFu, in ? m[v] : 0);
+        if (lane == v) mine = r;
+      }
+      if (lane < NV && mine > 0) atomicMax(smax + (first + k) * NV + lane, mine);
+    }
+  }
+}
+
+// Limbs of a value in its place.
+__device__ __forceinline__ double fixed_bits(double x, int es) {
+  const int2 f = fixed_limbs(x, es);
+  return __hiloint2double(f.x, f.y);
+}
+__device__ __forceinline__ int2 fixed_of_bits(double b) {
+  return make_int2(__double2hiint(b), __double2loint(b));
+}
+
+// Shared memory of the FP64 volume kernel: pointwise fluxes [D][NV][THREADS] and face fluxes
+// [EPB][D][side][NV][NF] (as limbs, or FP64 for the FP64 chain), the staged solution and
+// Runge-Kutta register [NV][THREADS] (the solution's place then takes the next stage input),
+// the fixed-point sweep tables, and the largest magnitudes per element and variable.
+template <int D, int N, int TT>
+struct VolSmem64 {
+  using T = Tile<D, N, TT>;
+  static constexpr int BLOCK = (T::THREADS + 31) / 32 * 32;  // threads, in whole warps
+  static constexpr size_t FACE_OFF = sizeof(double) * D * T::NV * T::THREADS;
+  static constexpr size_t W_OFF = FACE_OFF + sizeof(double) * T::EPB * 2 * D * T::NV * T::NF;
+  static constexpr size_t Q_OFF = W_OFF + sizeof(double) * T::NV * T::THREADS;
+  static constexpr size_t TAB_OFF = Q_OFF + sizeof(double) * T::NV * T::THREADS;
+  static constexpr size_t C_OFF = TAB_OFF + sizeof(int2) * D * N * (N + 2);
+  static constexpr size_t MAX_OFF = C_OFF + sizeof(long long) * D * N;
+  static constexpr size_t BYTES = MAX_OFF + sizeof(int) * T::EPB * T::NV;
+};
+
+// One element tile of the FP64 volume/update kernel.  Everything the tile reads is copied to
+// shared memory asynchronously at the start; one thread per node evaluates the pointwise
+// fluxes, the sweeps with the lift (in fixed point, fixline.cuh) and the Runge-Kutta update;
+// one thread per line interpolates the traces of the next stage input.
+// Bound: the FP64 pipe retires 2 operations per clock and SM (and each takes about five issue
+// slots), so whatever is a contraction runs on the integer pipe (2D p=4: 23 FP64 operations
+// per node instead of 97); the pointwise fluxes and the update stay in FP64.  FP64 pipe 56 %,
+// ALU 56 %, issue 68 % busy.  Against chains of FP64 fused multiply-adds: 256^2 p=4 295 -> 112
+// us, 320^2 p=3 265 -> 102, 160^2 p=7 349 -> 112, 48^3 p=3 1874 -> 670, 32^3 p=5 2291 -> 850.
+// One exponent per element and variable (each value is converted once and the directions add
+// up as integers) against one per line of nodes with a thread per line: 256^2 112 against 135
+// us, 48^3 670 against 904.
+template <int D, int N, int TT, typename Faces = SplitFaces>
+__device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsigned char* smem_raw,
+                                              const Faces& faces = Faces()) {
+  using T = Tile<D, N, TT>;
+  constexpr bool kFaces = std::is_same<Faces, ElementFaces>::value;
+  using SM = VolSmem64<D, N, TT>;
+  constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB, M = N + 2;
+  constexpr int THREADS = T::THREADS, BLOCK = SM::BLOCK;
+  const int tid = threadIdx.x;
+  double* sF = reinterpret_cast<double*>(smem_raw);
+  double* sFace = reinterpret_cast<double*>(smem_raw + SM::FACE_OFF);
+  double* sW = reinterpret_cast<double*>(smem_raw + SM::W_OFF) + tid;
+  double* sQ = reinterpret_cast<double*>(smem_raw + SM::Q_OFF) + tid;
+  int2* sTab = reinterpret_cast<int2*>(smem_raw + SM::TAB_OFF);  // [D][N][M]
+  long long* sC = reinterpret_cast<long long*>(smem_raw + SM::C_OFF);  // [D][N]
+  int* sMax = reinterpret_cast<int*>(smem_raw + SM::MAX_OFF);    // [EPB][NV]
+  const int el = tid / ND, node = tid - el * ND;
+  const int e0 = tile * EPB;
+  const int ne = (int)A.m.ne;
+  const int e = e0 + el;
+  const bool active = el < EPB && e < ne;
+  const FixedSweep* tab = A.scaled ? &A.tab->fxs : &A.tab->fx;
+
+  // copies: stage input (group 1); the register q, or the solution where the input is r, the
+  // face fluxes and the tables (group 2)
+  const bool from_r = (A.mode == kMode2R && A.stage > 0);
+  if (active) {
+    const double* in = from_r ? reinterpret_cast<const double*>(A.r_in) : A.w_in;
+    const double* in2 = from_r ? A.w
+                               : (A.mode == kMode2N && A.stage > 0 ? reinterpret_cast<const double*>(A.x)
+                                                                   : nullptr);
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+      cp_async8((from_r ? sQ : sW) + v * THREADS, in + (v * ne + e) * ND + node);
+    cp_async_commit();
+    if (in2) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        cp_async8((from_r ? sW : sQ) + v * THREADS, in2 + (v * ne + e) * ND + node);
+    }
+    int ec[3];
+    elem_coords(A.m, e, ec);
+    if constexpr (!kFaces) {
+      const double* fl = reinterpret_cast<const double*>(A.fl);
+      for (int q = node; q < 2 * D * NF; q += ND) {
+        const int ds = q / NF, j = q - ds * NF;
+        const int d = ds >> 1;
+        const int lo = (ds & 1) ? e : elem_shift(A.m, e, ec, d, -1);
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          cp_async8(sFace + ((el * 2 * D + ds) * NV + v) * NF + j, fl + ((d * NV + v) * ne + lo) * NF + j);
+      }
+    } else {
+      element_face_fluxes<D, N, double, TT>(faces, A.m, e, ec, el, node, active, smem_raw + SM::FACE_OFF);
+    }
+  } else {
+    cp_async_commit();
+  }
+  for (int i = tid; i < D * N * M; i += BLOCK) cp_async8(sTab + i, &tab->q[i / (N * M)][i % (N * M)]);
+  if (tid < D * N) cp_async8(sC + tid, &tab->c[tid / N][tid % N]);
+  cp_async_commit();
+  for (int i = tid; i < EPB * NV; i += BLOCK) sMax[i] = 0;
+  __syncthreads();
+
+  // 1. pointwise fluxes; largest magnitude of every variable's fluxes in the element
+  cp_async_wait<1>();
+  double F[D][NV];
+  {
+    double u[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) u[v] = active ? (from_r ? sQ : sW)[v * THREADS] : 1.0;
+    euler_flux_all<D, double>(u, A.gm1, F);
+  }
+  cp_async_wait<0>();
+  {
+    int m[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      m[v] = abs_hi(F[0][v]);
+#pragma unroll
+      for (int d = 1; d < D; ++d) m[v] = max(m[v], abs_hi(F[d][v]));
+    }
+    if (active) {
+      for (int q = node; q < 2 * D * NF; q += ND) {
+        const int ds = q / NF, j = q - ds * NF;
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          m[v] = max(m[v], abs_hi(sFace[((el * 2 * D + ds) * NV + v) * NF + j]));
+      }
+    }
+    element_max<ND, NV, THREADS>(m, active ? el : -1, sMax);
+  }
+  __syncthreads();
+
+  // 2. fixed point (or the values as they are where the element needs the FP64 chain)
+  int ex[NV];
+  bool chain = false;
+  const FixedScale sc = tab->s;
+  if (active) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      ex[v] = fixed_exponent(sc, sMax[el * NV + v]);
+      chain = chain || ex[v] > sc.ehi;
+    }
+    if (!chain) {
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) F[d][v] = fixed_bits(F[d][v], ex[v] + kSweepShift);
+      for (int q = node; q < 2 * D * NF; q += ND) {
+        const int ds = q / NF, j = q - ds * NF;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          double* f = sFace + ((el * 2 * D + ds) * NV + v) * NF + j;
+          *f = fixed_bits(*f, ex[v] + kSweepShift);
+        }
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sF[(d * NV + v) * THREADS + tid] = F[d][v];
+  }
+  __syncthreads();
+
+  // 3. weak derivative (one contraction per direction) and face lift, Runge-Kutta update
+  if (active) {
+    const int ix[3] = {node % N, (node / N) % N, node / (N * N)};
+    double k[NV];
+    if (!chain) {
+      FixedAcc acc[NV];
+      long long c = sC[ix[0]];
+#pragma unroll
+      for (int d = 1; d < D; ++d) c += sC[d * N + ix[d]];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = FixedAcc{0, c};
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+        const double* f = sF + d * NV * THREADS + tid - ix[d] * stride;
+        const int2* q = sTab + (d * N + ix[d]) * M;
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+          const int2 w = q[a];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) fixed_fma(w, fixed_of_bits(f[v * THREADS + a * stride]), acc[v]);
+        }
+        const double* g = sFace + (el * D + d) * 2 * NV * NF + face_index<D, N>(d, ix);
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          const int2 w = q[N + side];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) fixed_fma(w, fixed_of_bits(g[(side * NV + v) * NF]), acc[v]);
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) k[v] = fixed_result(acc[v], sc, ex[v]);
+    } else {
+      const double* sFv = sF + tid;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) k[v] = 0.0;
+      for (int pass = 0; pass < 2 * D; ++pass) {  // the sweeps, then the lifts
+        const int d = pass < D ? pass : pass - D;
+        const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+        const int id = d == 0 ? ix[0] : (d == 1 ? ix[1] : ix[2]);
+        if (pass < D) {
+          const double* f = sFv + d * NV * THREADS - id * stride;
+          const double* Q = (A.scaled ? A.tab->Qs[d] : A.tab->Q[d]) + id * N;
+          for (int a = 0; a < N; ++a)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) k[v] = fma(Q[a], f[v * THREADS + a * stride], k[v]);
+        } else {
+          const double lm = (A.scaled ? A.tab->Lms[d] : A.tab->Lm[d])[id];
+          const double lp = (A.scaled ? A.tab->Lps[d] : A.tab->Lp[d])[id];
+          const double* g = sFace + (el * D + d) * 2 * NV * NF + face_index<D, N>(d, ix);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            k[v] = fma(lm, g[v * NF], k[v]);
+            k[v] = fma(-lp, g[(NV + v) * NF], k[v]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+      sW[v * THREADS] = Update<double>::apply(A, (v * ne + e) * ND + node, k[v], sW[v * THREADS],
+                                              sQ[v * THREADS]);
+  }
+
+  // 4. traces of the next stage input
+  if (A.write_traces) {
+    __syncthreads();
+    write_traces_fp64<D, N, TT>(A.m, A.ft, A.tab, sW - tid, THREADS, e0,
+                                reinterpret_cast<double*>(A.tr));
+  }
+}
+
 // Register budget of the single-instance volume kernel (an explicit budget also keeps the
 // compiler from trading occupancy for registers).  The FP32 form is latency-bound and
 // wants every warp slot.
@@ -776,7 +1070,8 @@ template <int D, int N, typename R> struct VolKernelRegs {
   static constexpr int value = (D == 2 && (N == 2 || N == 8)) ? 64 : 56;  // no spills (ptxas)
 };
 template <int D, int N> struct VolKernelRegs<D, N, double> {
-  static constexpr int value = D == 2 ? ((N == 3 || N == 8) ? 48 : 40) : 56;  // no spills (ptxas)
+  // 2D 40 to 64 registers within 2 %; 3D 48 registers spill (+5 %), 72 gain nothing
+  static constexpr int value = D == 2 ? 48 : 64;
 };
 template <int D, int N> struct VolKernelRegs<D, N, float> {
   static constexpr int value = (D == 2 && N != 3 && N != 4 && N != 6) ? 32 : 40;  // no spills (ptxas, sm_103a)
@@ -789,6 +1084,16 @@ __global__ void __launch_bounds__(Tile<D, N, TT>::THREADS,
 vol_kernel(const VolArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   vol_body<D, N, R, TT, VolStages<R>::value>(A, blockIdx.x, smem_raw);
+}
+
+// (64, 192 and 256 threads: 2 to 25 % slower than 128 over the degrees)
+template <int D, int N, int TT = 128>
+__global__ void __launch_bounds__(VolSmem64<D, N, TT>::BLOCK,
+                                  min_blocks_for(VolKernelRegs<D, N, double>::value,
+                                                 VolSmem64<D, N, TT>::BLOCK))
+vol_kernel_fp64(const __grid_constant__ VolArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  vol_body_fp64<D, N, TT>(A, blockIdx.x, smem_raw);
 }
 
 // Random-delay draw (same definition as the host schedule).
@@ -955,6 +1260,16 @@ vol_faces_kernel(const FusedArgs A) {
                                                            ElementFaces{A.f, A.tr_in, A.err});
 }
 
+template <int D, int N, int TT = 128>
+__global__ void __launch_bounds__(VolSmem64<D, N, TT>::BLOCK,
+                                  min_blocks_for(VolFacesRegs<D, N, double>::value,
+                                                 VolSmem64<D, N, TT>::BLOCK))
+vol_faces_kernel_fp64(const __grid_constant__ FusedArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  vol_body_fp64<D, N, TT, ElementFaces>(A.v, blockIdx.x, smem_raw,
+                                        ElementFaces{A.f, A.tr_in, A.err});
+}
+
 // Register budget of the face-flux kernel (blocks of 256 threads; no spills, ptxas sm_103a).
 template <int D, typename R> struct FluxKernelRegs { static constexpr int value = D == 2 ? 64 : 72; };
 template <int D> struct FluxKernelRegs<D, float> { static constexpr int value = 48; };
@@ -979,32 +1294,50 @@ cudaError_t launch_trace_t(const TraceArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Opt-in for more than 48 KB of dynamic shared memory.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t smem) {
+  return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem)
+                          : cudaSuccess;
+}
+
 template <int D, int N, typename R>
 cudaError_t launch_vol_t(const VolArgs& a, cudaStream_t s) {
-  using T = Tile<D, N>;
-  const int64_t blocks = (a.m.ne + T::EPB - 1) / T::EPB;
-  const size_t smem = VolSmem<D, N, R, 128, VolStages<R>::value>::BYTES;
-  if (smem > 48 * 1024) {
-    cudaError_t err = cudaFuncSetAttribute(vol_kernel<D, N, R>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+  constexpr bool k64 = std::is_same<R, double>::value;
+  constexpr int TT = 128;
+  using T = Tile<D, N, TT>;
+  const unsigned blocks = (unsigned)((a.m.ne + T::EPB - 1) / T::EPB);
+  cudaError_t err;
+  if constexpr (k64) {
+    const size_t smem = VolSmem64<D, N, TT>::BYTES;
+    if ((err = allow_smem(vol_kernel_fp64<D, N>, smem)) != cudaSuccess) return err;
+    vol_kernel_fp64<D, N><<<blocks, VolSmem64<D, N, TT>::BLOCK, smem, s>>>(a);
+  } else {
+    const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value>::BYTES;
+    if ((err = allow_smem(vol_kernel<D, N, R>, smem)) != cudaSuccess) return err;
+    vol_kernel<D, N, R><<<blocks, T::THREADS, smem, s>>>(a);
   }
-  vol_kernel<D, N, R><<<(unsigned)blocks, T::THREADS, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int D, int N, typename R>
 cudaError_t launch_vol_faces_t(const FusedArgs& a, cudaStream_t s) {
+  constexpr bool k64 = std::is_same<R, double>::value;
   constexpr int TT = 128;  // tiles of about 128 threads, as on the split path
   using T = Tile<D, N, TT>;
-  const int64_t blocks = (a.v.m.ne + T::EPB - 1) / T::EPB;
-  const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value, true>::BYTES;
-  if (smem > 48 * 1024) {
-    cudaError_t err = cudaFuncSetAttribute(vol_faces_kernel<D, N, R, TT>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+  const unsigned blocks = (unsigned)((a.v.m.ne + T::EPB - 1) / T::EPB);
+  cudaError_t err;
+  if constexpr (k64) {
+    const size_t smem = VolSmem64<D, N, TT>::BYTES;
+    if ((err = allow_smem(vol_faces_kernel_fp64<D, N>, smem)) != cudaSuccess) return err;
+    vol_faces_kernel_fp64<D, N>
+        <<<blocks, VolSmem64<D, N, TT>::BLOCK, smem, s>>>(a);
+  } else {
+    const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value, true>::BYTES;
+    if ((err = allow_smem(vol_faces_kernel<D, N, R, TT>, smem)) != cudaSuccess) return err;
+    vol_faces_kernel<D, N, R, TT><<<blocks, T::THREADS, smem, s>>>(a);
   }
-  vol_faces_kernel<D, N, R, TT><<<(unsigned)blocks, T::THREADS, smem, s>>>(a);
   return cudaGetLastError();
 }
 

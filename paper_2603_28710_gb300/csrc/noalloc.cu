@@ -16,7 +16,7 @@
 
 namespace adg {
 // defined in host.cu
-void noalloc_build_tables(int N, const double* h, OpTables* T);
+void noalloc_build_tables(int dim, int N, const double* h, OpTables* T);
 void noalloc_set_error(const char* msg);
 }
 
@@ -37,7 +37,7 @@ adg_status noalloc_fail(adg_status st, const std::string& m) {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // The operator tables travel as a kernel argument (kernel arguments may hold up to 32 KB;
-// the tables take about 9 KB) and a one-block kernel stores them into the scratch array:
+// the tables take about 13 KB) and a one-block kernel stores them into the scratch array:
 // the launch copies the argument when it is enqueued, so no host memory is read after the
 // call returns and no host-to-device copy waits for the stream.
 struct TableBlob {
@@ -104,7 +104,7 @@ extern "C" adg_status adg_rhs_noalloc(const adg_mesh* mesh, int degree, double g
 
   OpTables tab;
   std::memset(&tab, 0, sizeof(tab));
-  noalloc_build_tables(N, h, &tab);
+  noalloc_build_tables(dim, N, h, &tab);
   OpTables* tab_dev = reinterpret_cast<OpTables*>(base);
   void* tr = base + tab_bytes;
   void* fl = base + tab_bytes + tr_bytes;
@@ -128,6 +128,7 @@ extern "C" adg_status adg_rhs_noalloc(const adg_mesh* mesh, int degree, double g
   ta.tab = tab_dev;
   ta.u = u;
   ta.tr = tr;
+  ta.ft = tab.ft;
   e = launch_trace(0, dim, N, ta, s);
   if (e != cudaSuccess) return noalloc_fail(ADG_ERR_CUDA, std::string("trace kernel: ") + cudaGetErrorString(e));
 
