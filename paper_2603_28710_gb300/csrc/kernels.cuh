@@ -117,27 +117,36 @@ __device__ __forceinline__ void euler_flux_all(const R (&w)[D + 2], R gm1, R (&F
   }
 }
 
-// Flux column along e_d and |u|^2 + c^2 of one trace state (d is a runtime direction;
+// Velocity along e_d, pressure and |u|^2 + c^2 of one trace state (d is a runtime direction;
 // selects instead of indexing keep everything in registers).
 template <int D, typename R>
-__device__ __forceinline__ void side_flux(const R (&w)[D + 2], int d, R gamma, R gm1,
-                                          R (&fd)[D + 2], R& s2) {
+__device__ __forceinline__ void side_state(const R (&w)[D + 2], int d, R gamma, R gm1, R& ud, R& p,
+                                           R& s2) {
   const R irho = r_rcp(w[0]);
-  R k2 = R(0.0f), ud = R(0.0f), md = w[1];
+  R k2 = R(0.0f);
+  ud = R(0.0f);
 #pragma unroll
   for (int c = 0; c < D; ++c) {
     const R uc = w[1 + c] * irho;
     k2 = r_fma(w[1 + c], uc, k2);  // rho |u|^2
-    if (c == d) {
-      ud = uc;
-      md = w[1 + c];
-    }
+    if (c == d) ud = uc;
   }
-  const R p = gm1 * sub_half(w[D + 1], k2);  // (gamma - 1) (E - rho |u|^2 / 2)
-  s2 = r_fma(gamma, p, k2) * irho;           // |u|^2 + gamma p / rho
-  fd[0] = md;
+  p = gm1 * sub_half(w[D + 1], k2);  // (gamma - 1) (E - rho |u|^2 / 2)
+  s2 = r_fma(gamma, p, k2) * irho;   // |u|^2 + gamma p / rho
+}
+
+// Flux column along e_d and |u|^2 + c^2 of one trace state.
+template <int D, typename R>
+__device__ __forceinline__ void side_flux(const R (&w)[D + 2], int d, R gamma, R gm1,
+                                          R (&fd)[D + 2], R& s2) {
+  R ud, p;
+  side_state<D, R>(w, d, gamma, gm1, ud, p, s2);
+  fd[0] = w[1];
 #pragma unroll
-  for (int c = 0; c < D; ++c) fd[1 + c] = c == d ? r_fma(w[1 + c], ud, p) : w[1 + c] * ud;
+  for (int c = 0; c < D; ++c) {
+    if (c == d) fd[0] = w[1 + c];
+    fd[1 + c] = c == d ? r_fma(w[1 + c], ud, p) : w[1 + c] * ud;
+  }
   fd[D + 1] = (w[D + 1] + p) * ud;
 }
 
@@ -150,27 +159,51 @@ template <int D, typename R>
 __device__ __forceinline__ void llf_flux(const R (&wm)[D + 2], const R (&wp)[D + 2], int d,
                                          R gamma, R gm1, R (&f)[D + 2]) {
   constexpr int NV = D + 2;
-  R fm[NV], fp[NV], sm, sp;
-  if constexpr (std::is_same<R, df64>::value) {
-    // FP32 pairs: both sides in the two lanes of packed FP32x2 instructions
-    df64x2 w2[NV], f2[NV], s2;
+  if constexpr (std::is_same<R, double>::value) {
+    // Bound by the FP64 pipe, 2D 45 and 3D 53 operations (from about 78 and 81): the square
+    // root takes 5, the larger speed is found by integer comparison, and the two sides'
+    // products are summed as they are formed.  256^2 p=4: 81 -> 68 us per launch; 48^3 p=3:
+    // 677 -> 552 us.
+    double um, up, pm, pp, sm, sp;
+    side_state<D, double>(wm, d, gamma, gm1, um, pm, sm);
+    side_state<D, double>(wp, d, gamma, gm1, up, pp, sp);
+    const double lam = half_sqrt(speed_max(sm, sp)), psum = pm + pp;
+    double mm = wm[1], mp = wp[1];  // normal momentum
 #pragma unroll
-    for (int v = 0; v < NV; ++v) w2[v] = df64x2_of(wm[v], wp[v]);
-    side_flux<D, df64x2>(w2, d, df64x2_of(gamma, gamma), df64x2_of(gm1, gm1), f2, s2);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      fm[v] = df64x2_lane(f2[v], 0);
-      fp[v] = df64x2_lane(f2[v], 1);
+    for (int c = 1; c < D; ++c) {
+      mm = c == d ? wm[1 + c] : mm;
+      mp = c == d ? wp[1 + c] : mp;
     }
-    sm = df64x2_lane(s2, 0);
-    sp = df64x2_lane(s2, 1);
-  } else {
-    side_flux<D, R>(wm, d, gamma, gm1, fm, sm);
-    side_flux<D, R>(wp, d, gamma, gm1, fp, sp);
-  }
-  const R lam = scale_pow2(r_sqrt(r_max(sm, sp)), 0.5f);
+    f[0] = fma(lam, wm[0] - wp[0], mm + mp);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) f[v] = r_fma(lam, wm[v] - wp[v], fm[v] + fp[v]);
+    for (int c = 0; c < D; ++c) {
+      const double s = fma(wm[1 + c], um, c == d ? psum : 0.0);
+      f[1 + c] = fma(lam, wm[1 + c] - wp[1 + c], fma(wp[1 + c], up, s));
+    }
+    f[D + 1] = fma(lam, wm[D + 1] - wp[D + 1], fma(wp[D + 1] + pp, up, (wm[D + 1] + pm) * um));
+  } else {
+    R fm[NV], fp[NV], sm, sp;
+    if constexpr (std::is_same<R, df64>::value) {
+      // FP32 pairs: both sides in the two lanes of packed FP32x2 instructions
+      df64x2 w2[NV], f2[NV], s2;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w2[v] = df64x2_of(wm[v], wp[v]);
+      side_flux<D, df64x2>(w2, d, df64x2_of(gamma, gamma), df64x2_of(gm1, gm1), f2, s2);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        fm[v] = df64x2_lane(f2[v], 0);
+        fp[v] = df64x2_lane(f2[v], 1);
+      }
+      sm = df64x2_lane(s2, 0);
+      sp = df64x2_lane(s2, 1);
+    } else {
+      side_flux<D, R>(wm, d, gamma, gm1, fm, sm);
+      side_flux<D, R>(wp, d, gamma, gm1, fp, sp);
+    }
+    const R lam = scale_pow2(r_sqrt(r_max(sm, sp)), 0.5f);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) f[v] = r_fma(lam, wm[v] - wp[v], fm[v] + fp[v]);
+  }
 }
 
 // Transverse coordinates of face node j of a face normal to d -> base node index of the
@@ -1270,14 +1303,19 @@ vol_faces_kernel_fp64(const __grid_constant__ FusedArgs A) {
                                         ElementFaces{A.f, A.tr_in, A.err});
 }
 
-// Register budget of the face-flux kernel (blocks of 256 threads; no spills, ptxas sm_103a).
+// Face-flux blocks of 64 threads: a small mesh spreads over more SMs (the FP64 pipe of an SM
+// works off one warp per 64 clocks and instruction whatever its lanes hold; 16^2 p=2 17.4 ->
+// 14.7 us per stage against 256 threads), and the pair form's last wave is fuller (256^2 p=4
+// 29.6 -> 27.3 us, 48^3 p=3 217 -> 203 us).
+constexpr int kFluxThreads = 64;
+// Register budget of the face-flux kernel (no spills, ptxas sm_103a).
 template <int D, typename R> struct FluxKernelRegs { static constexpr int value = D == 2 ? 64 : 72; };
 template <int D> struct FluxKernelRegs<D, float> { static constexpr int value = 48; };
 template <int D> struct FluxKernelRegs<D, df64> { static constexpr int value = 64; };
 
 // grid: x over (element, face node) of one direction, y = direction d
 template <int D, int N, typename R>
-__global__ void __launch_bounds__(256, min_blocks_for(FluxKernelRegs<D, R>::value, 256))
+__global__ void __launch_bounds__(kFluxThreads, min_blocks_for(FluxKernelRegs<D, R>::value, kFluxThreads))
 flux_kernel(const FluxArgs A) {
   flux_body<D, N, R>(A, blockIdx.x, blockIdx.y);
 }
@@ -1331,8 +1369,7 @@ cudaError_t launch_vol_faces_t(const FusedArgs& a, cudaStream_t s) {
   if constexpr (k64) {
     const size_t smem = VolSmem64<D, N, TT>::BYTES;
     if ((err = allow_smem(vol_faces_kernel_fp64<D, N>, smem)) != cudaSuccess) return err;
-    vol_faces_kernel_fp64<D, N>
-        <<<blocks, VolSmem64<D, N, TT>::BLOCK, smem, s>>>(a);
+    vol_faces_kernel_fp64<D, N><<<blocks, VolSmem64<D, N, TT>::BLOCK, smem, s>>>(a);
   } else {
     const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value, true>::BYTES;
     if ((err = allow_smem(vol_faces_kernel<D, N, R, TT>, smem)) != cudaSuccess) return err;
@@ -1345,8 +1382,8 @@ template <int D, int N, typename R>
 cudaError_t launch_flux_t(const FluxArgs& a, cudaStream_t s) {
   constexpr int NF = IPow<N, D - 1>::value;
   const int64_t per_dir = a.m.ne * NF;
-  dim3 grid((unsigned)((per_dir + 255) / 256), D);
-  flux_kernel<D, N, R><<<grid, 256, 0, s>>>(a);
+  dim3 grid((unsigned)((per_dir + kFluxThreads - 1) / kFluxThreads), D);
+  flux_kernel<D, N, R><<<grid, kFluxThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
