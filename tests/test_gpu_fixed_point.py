@@ -137,3 +137,22 @@ def test_nonfinite_values_spread_along_lines(dim, n_elem, p, bad):
     far = np.abs(k.reshape(u.shape) - clean) <= bound
     assert far.reshape(full)[:, ~hit].all()
     s.close()
+
+
+@pytest.mark.parametrize("exponent", [-290, -200, -37, 0, 37, 200, 290])
+@pytest.mark.parametrize("dim,n_elem,p", [(2, (5, 3), 3), (3, (3, 2, 2), 2)])
+def test_signal_speeds_of_any_magnitude(dim, n_elem, p, exponent):
+    # a gas at rest with energies of 10^exponent: the face flux's square root (an FP32 seed on
+    # the scaled argument) over the exponent range, the momentum fluxes and the dissipation of
+    # the density with it
+    s, o = solver(dim, n_elem, p), oracle(dim, n_elem, p)
+    u = random_state(s.shape, dim, seed=600 + p)
+    u[1:1 + dim] = 0.0
+    u[dim + 1] *= 10.0 ** exponent
+    kg, ko = s.rhs(u), o.rhs(u)
+    h = [(1.0, 2.0, 3.0)[d] / n_elem[d] for d in range(dim)]
+    with np.errstate(over="ignore"):
+        bound = 256 * EPS * sum_scale(u, dim, p, n_elem, h)[:, :, None]
+    rows = slice(0, 1 + dim if exponent >= 200 else dim + 2)  # (energy row: 1e290 * 1e145)
+    assert (np.abs(kg - ko) <= bound)[rows].all(), (np.abs(kg - ko) / bound)[rows].max()
+    s.close()
