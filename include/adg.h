@@ -340,7 +340,8 @@ void adg_batch_destroy(adg_batch* b);
 int adg_mlp_num_params(void);
 /* Mean squared error over n samples (x[n][4], target[n]): ADDS d(loss)/d(params) to grad
  * (FP32, one value per parameter) and the loss to *loss (one float).  Forward and backward
- * pass in FP32 arithmetic with the BF16 weights. */
+ * pass to FP32 accuracy with the BF16 weights (products of the hidden layer on the tensor
+ * cores, FP32 values as three BF16 terms each). */
 adg_status adg_mlp_grad(const uint16_t* params_bf16, const float* x, const float* target,
                         int64_t n, float* grad, float* loss, void* cuda_stream);
 /* y[n] = MLP(x[n][4]).  The hidden 64 x 64 layer runs on the tensor cores (BF16 MMA with

@@ -1,8 +1,8 @@
 // Learned ghost-trace predictor: a small MLP, 4 inputs -> 64 -> 64 -> 1, tanh hidden
 // activations, BF16 weights read into FP32 and FP32 accumulation everywhere.  Kernels for
-// the mean-squared-error gradient of a sample set (forward + backward, FP32 pipe), an Adam
-// step on FP32 master weights that refreshes their BF16 copy, and inference (the hidden
-// layer on the tensor cores).
+// the mean-squared-error gradient of a sample set (forward + backward) and inference, with the
+// hidden layer's products on the tensor cores, and an Adam step on FP32 master weights that
+// refreshes their BF16 copy.
 //
 // Parameter layout (kMlpParams = 4545 values):
 //   W1[64][4] | b1[64] | W2[64][64] | b2[64] | w3[64] | b3
@@ -19,125 +19,14 @@ void noalloc_set_error(const char* msg);
 
 namespace {
 
-constexpr int kSamples = 128;   // samples per chunk (one per thread)
-constexpr int kPad = kSamples + 1;  // row stride of the per-sample tables (no bank conflicts)
-
-// shared memory: weights | X[4][kPad] | H1[64][kPad] | H2[64][kPad] | DZ2[64][kPad] | DZ1[64][kPad] | DY[kPad]
-constexpr int kSmemFloats = 4548 + 4 * kPad + 4 * 64 * kPad + kPad;
-
-__global__ void __launch_bounds__(kSamples)
-mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
-                const float* __restrict__ t, int n, float inv_n, float* __restrict__ grad,
-                float* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* W = sm;
-  float* X = W + 4548;
-  float* H1 = X + 4 * kPad;
-  float* H2 = H1 + 64 * kPad;
-  float* DZ2 = H2 + 64 * kPad;
-  float* DZ1 = DZ2 + 64 * kPad;
-  float* DY = DZ1 + 64 * kPad;
-  const int tid = threadIdx.x;
-  for (int i = tid; i < kMlpParams; i += blockDim.x) W[i] = bf16_to_float(pbf[i]);
-  // each thread owns gradient entries tid, tid + 128, ... (36 of them at most)
-  constexpr int kOwn = (kMlpParams + kSamples - 1) / kSamples;
-  float gacc[kOwn];
-#pragma unroll
-  for (int k = 0; k < kOwn; ++k) gacc[k] = 0.0f;
-  float lacc = 0.0f;
-  __syncthreads();
-  const int chunks = (n + kSamples - 1) / kSamples;
-  for (int c = blockIdx.x; c < chunks; c += gridDim.x) {
-    const int s = c * kSamples + tid;
-    const bool valid = s < n;
-    float xi[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      xi[i] = valid ? x[(size_t)s * 4 + i] : 0.0f;
-      X[i * kPad + tid] = xi[i];
-    }
-    // forward
-    for (int j = 0; j < 64; ++j) {
-      float z = W[kB1 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) z = fmaf(W[kW1 + j * 4 + i], xi[i], z);
-      H1[j * kPad + tid] = tanhf(z);
-    }
-    float y = W[kB3];
-    for (int j = 0; j < 64; ++j) {
-      float z = W[kB2 + j];
-      for (int i = 0; i < 64; ++i) z = fmaf(W[kW2 + j * 64 + i], H1[i * kPad + tid], z);
-      const float h = tanhf(z);
-      H2[j * kPad + tid] = h;
-      y = fmaf(W[kW3 + j], h, y);
-    }
-    const float r = valid ? (y - t[s]) : 0.0f;
-    lacc = fmaf(r * r, inv_n, lacc);
-    const float dy = 2.0f * r * inv_n;
-    DY[tid] = dy;
-    // backward
-    for (int j = 0; j < 64; ++j) {
-      const float h = H2[j * kPad + tid];
-      DZ2[j * kPad + tid] = dy * W[kW3 + j] * (1.0f - h * h);
-    }
-    for (int i = 0; i < 64; ++i) {
-      float dh = 0.0f;
-      for (int j = 0; j < 64; ++j) dh = fmaf(W[kW2 + j * 64 + i], DZ2[j * kPad + tid], dh);
-      const float h = H1[i * kPad + tid];
-      DZ1[i * kPad + tid] = dh * (1.0f - h * h);
-    }
-    __syncthreads();
-    // gradient contributions of this chunk, summed over its samples
-#pragma unroll
-    for (int k = 0; k < kOwn; ++k) {
-      const int e = tid + k * kSamples;
-      if (e >= kMlpParams) break;
-      float acc = 0.0f;
-      if (e < kB1) {                       // W1[j][i]
-        const int j = e >> 2, i = e & 3;
-        for (int q = 0; q < kSamples; ++q) acc = fmaf(DZ1[j * kPad + q], X[i * kPad + q], acc);
-      } else if (e < kW2) {                // b1[j]
-        const int j = e - kB1;
-        for (int q = 0; q < kSamples; ++q) acc += DZ1[j * kPad + q];
-      } else if (e < kB2) {                // W2[j][i]
-        const int j = (e - kW2) >> 6, i = (e - kW2) & 63;
-        for (int q = 0; q < kSamples; ++q) acc = fmaf(DZ2[j * kPad + q], H1[i * kPad + q], acc);
-      } else if (e < kW3) {                // b2[j]
-        const int j = e - kB2;
-        for (int q = 0; q < kSamples; ++q) acc += DZ2[j * kPad + q];
-      } else if (e < kB3) {                // w3[j]
-        const int j = e - kW3;
-        for (int q = 0; q < kSamples; ++q) acc = fmaf(DY[q], H2[j * kPad + q], acc);
-      } else {                             // b3
-        for (int q = 0; q < kSamples; ++q) acc += DY[q];
-      }
-      gacc[k] += acc;
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int k = 0; k < kOwn; ++k) {
-    const int e = tid + k * kSamples;
-    if (e < kMlpParams) atomicAdd(&grad[e], gacc[k]);
-  }
-  // block-reduce the loss
-  __shared__ float red[kSamples];
-  red[tid] = lacc;
-  __syncthreads();
-  for (int st = kSamples / 2; st > 0; st >>= 1) {
-    if (tid < st) red[tid] += red[tid + st];
-    __syncthreads();
-  }
-  if (tid == 0) atomicAdd(loss, red[0]);
-}
-
-// ---- inference on the tensor cores --------------------------------------------------
-// The 64 x 64 hidden layer of a tile of 16 samples is a [16 x 64] x [64 x 64] product: warp-
-// level BF16 MMAs (mma.sync m16n8k16, FP32 accumulation).  The BF16 weights enter exactly;
-// the FP32 activations of the first layer are split into three BF16 terms
-// h = h0 + h1 + h2 (each the BF16 rounding of what the previous terms leave; residual below
-// 2^-24 |h|), so the product keeps FP32 accuracy at three MMAs per k-step.  The 4 -> 64
-// input layer, the tanh activations and the 64 -> 1 output layer stay on the FP32 pipe.
+// ---- BF16 tensor-core products of FP32 values ------------------------------------------
+// The 64 x 64 hidden layer of 16 samples is a [16 x 64] x [64 x 64] product: warp-level BF16
+// MMAs (mma.sync m16n8k16, FP32 accumulation).  The BF16 weights enter exactly; FP32 values are
+// split into three BF16 terms h = h0 + h1 + h2 (each the BF16 rounding of what the previous
+// terms leave; residual below 2^-24 |h|), so a product with the weights keeps FP32 accuracy
+// at three MMAs per k-step, and a product of two FP32 matrices at six (the terms of relative
+// size down to 2^-16; the rest is below 2^-24).  The 4 -> 64 input layer, the tanh
+// activations and the 64 -> 1 output layer stay on the FP32 pipe.
 //
 // Fragment layouts of mma.m16n8k16 (PTX ISA; g = lane / 4, t = lane % 4):
 //   A (16 x 16, row-major, 4 x b32 = 8 bf16): reg 0 = rows g, cols 2t, 2t+1; reg 1 = row g+8;
@@ -146,20 +35,20 @@ mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
 //     rows 2t+8, 2t+9
 //   C/D (16 x 8, f32): c0, c1 = row g, cols 2t, 2t+1; c2, c3 = row g+8
 
-__device__ __forceinline__ unsigned short bf16_bits_rn(float f) { return float_to_bf16(f); }
-
+// two values rounded to BF16 (nearest even), the first in the lower half
 __device__ __forceinline__ unsigned pack_bf16(float lo_col, float hi_col) {
-  return (unsigned)bf16_bits_rn(lo_col) | ((unsigned)bf16_bits_rn(hi_col) << 16);
+  unsigned r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi_col), "f"(lo_col));
+  return r;
 }
 
-// three-term BF16 split of two adjacent activations into three packed registers
+// three-term BF16 split of two adjacent values into three packed registers
 __device__ __forceinline__ void split3(float a, float b, unsigned& r0, unsigned& r1, unsigned& r2) {
-  const float a0 = bf16_to_float(bf16_bits_rn(a)), b0 = bf16_to_float(bf16_bits_rn(b));
-  const float a1r = a - a0, b1r = b - b0;  // exact (Sterbenz)
-  const float a1 = bf16_to_float(bf16_bits_rn(a1r)), b1 = bf16_to_float(bf16_bits_rn(b1r));
-  r0 = pack_bf16(a0, b0);
-  r1 = pack_bf16(a1, b1);
-  r2 = pack_bf16(a1r - a1, b1r - b1);
+  r0 = pack_bf16(a, b);
+  const float ar = a - __uint_as_float(r0 << 16);  // exact (Sterbenz)
+  const float br = b - __uint_as_float(r0 & 0xFFFF0000u);
+  r1 = pack_bf16(ar, br);
+  r2 = pack_bf16(ar - __uint_as_float(r1 << 16), br - __uint_as_float(r1 & 0xFFFF0000u));
 }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], unsigned b0,
@@ -171,6 +60,343 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// c += a b with the product rounded like an FP32 sum: the tensor cores add to their accumulator
+// with truncation, so a long sum is kept outside of it.
+__device__ __forceinline__ void mma_add(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  mma_bf16(p, a, b0, b1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) c[q] += p[q];
+}
+// Sum of products of a three-term FP32 fragment with BF16 weights: leading terms in `c`, the
+// others (2^-8 of them and less, where the truncation does not show) in `low`.
+__device__ __forceinline__ void mma_split(float (&c)[4], float (&low)[4], const unsigned (&a)[3][4],
+                                          unsigned b0, unsigned b1) {
+  mma_bf16(low, a[2], b0, b1);
+  mma_bf16(low, a[1], b0, b1);
+  mma_add(c, a[0], b0, b1);
+}
+
+// four 8 x 8 BF16 tiles from shared memory, transposed; lanes 8m..8m+7 hold the row addresses
+// of tile m (16 bytes each, 16-byte aligned)
+__device__ __forceinline__ void ldmatrix_trans(unsigned (&r)[4], const uint16_t* row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(row))
+               : "memory");
+}
+
+// First-layer activations tanh(W1 x + b1) of the 16-column block kk for rows g and g+8: h[row]
+// [columns c, c+1, c+8, c+9], c = 16 kk + 2t.  w: W1[64][4] | b1[64].
+__device__ __forceinline__ void first_layer(const float* w, const float (&x0)[4], const float (&x1)[4],
+                                            int kk, int t, float (&h)[2][4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = kk * 16 + 2 * t + (q & 1) + (q >> 1) * 8;
+    float z0 = w[kB1 + c], z1 = w[kB1 + c];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      z0 = fmaf(w[kW1 + c * 4 + i], x0[i], z0);
+      z1 = fmaf(w[kW1 + c * 4 + i], x1[i], z1);
+    }
+    h[0][q] = tanhf(z0);
+    h[1][q] = tanhf(z1);
+  }
+}
+
+// A fragments (three terms) of the values v[row][columns c, c+1, c+8, c+9]
+__device__ __forceinline__ void split_fragment(const float (&v)[2][4], unsigned (&a)[3][4]) {
+  split3(v[0][0], v[0][1], a[0][0], a[1][0], a[2][0]);
+  split3(v[1][0], v[1][1], a[0][1], a[1][1], a[2][1]);
+  split3(v[0][2], v[0][3], a[0][2], a[1][2], a[2][2]);
+  split3(v[1][2], v[1][3], a[0][3], a[1][3], a[2][3]);
+}
+
+// ---- gradient ------------------------------------------------------------------------
+// A block takes chunks of 128 samples, 16 per warp: forward pass, error and backward pass in
+// registers (z2 = h1 W2^T and dh1 = dz2 W2 on the tensor cores), the BF16 terms of h1 and dz2
+// and the FP32 dz1 into shared memory; then the block forms dW2 = dz2^T h1 on the tensor cores
+// (each warp a 16 x 32 part of it, its sum over the chunks in registers) and dW1, db1 on the
+// FP32 pipe.  Bound by latency at 8 warps per SM.  65536 samples with the Adam step: 219 -> 46 us
+// against one sample per thread with every product a chain of shared-memory operands; errors
+// against 64 bits unchanged.
+constexpr int kSamples = 128;   // samples per chunk
+constexpr int kGradThreads = 256;
+constexpr int kPitch = 72;      // BF16 row pitch: 16-byte rows, 8 rows in distinct banks
+constexpr int kZPitch = 65;     // FP32 row pitch of dz1
+
+struct GradSmem {
+  uint16_t h1[3][kSamples][kPitch];
+  uint16_t d2[3][kSamples][kPitch];
+  uint16_t w2[64][kPitch];   // [out][in]
+  uint16_t w2t[64][kPitch];  // [in][out]
+  float z1[kSamples][kZPitch];
+  float x[kSamples][4];
+  float w1[kW2];             // W1 | b1
+  float wo[kMlpParams - kB2];  // b2 | w3 | b3
+};
+
+__global__ void __launch_bounds__(kGradThreads)
+mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
+                const float* __restrict__ target, int n, float inv_n, float* __restrict__ grad,
+                float* __restrict__ loss) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  for (int i = tid; i < kW2; i += kGradThreads) S.w1[i] = bf16_to_float(pbf[i]);
+  for (int i = tid; i < kMlpParams - kB2; i += kGradThreads) S.wo[i] = bf16_to_float(pbf[kB2 + i]);
+  for (int i = tid; i < 64 * 64; i += kGradThreads) {
+    const uint16_t w = pbf[kW2 + i];
+    S.w2[i >> 6][i & 63] = w;
+    S.w2t[i & 63][i >> 6] = w;
+  }
+  // this thread's sums over all chunks: dW2 part; db2 and dw3 of the columns 8j + 2t + q; dW1
+  // and db1 of unit tid % 64 over a quarter of each chunk; db3 and the loss
+  float gw2[4][4], gb2[8][2], gw3[8][2], gw1[5], gb3 = 0.0f, lacc = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) gw2[i][q] = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) gb2[j][q] = gw3[j][q] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) gw1[i] = 0.0f;
+  const int m0 = (warp & 3) * 16, i0 = (warp >> 2) * 32;  // dW2 rows (out) and columns (in)
+  __syncthreads();
+
+  const int chunks = (n + kSamples - 1) / kSamples;
+  for (int c = blockIdx.x; c < chunks; c += gridDim.x) {
+    const int row0 = warp * 16 + g, row1 = row0 + 8;  // rows within the chunk
+    const int s0 = c * kSamples + row0, s1 = s0 + 8;
+    float x0[4], x1[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x0[i] = s0 < n ? x[(size_t)s0 * 4 + i] : 0.0f;
+      x1[i] = s1 < n ? x[(size_t)s1 * 4 + i] : 0.0f;
+    }
+    if (t == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        S.x[row0][i] = x0[i];
+        S.x[row1][i] = x1[i];
+      }
+    }
+    // forward
+    float f1[4][2][4];  // 1 - h1^2
+    float acc[8][4], low[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[j][q] = low[j][q] = 0.0f;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      float h[2][4];
+      first_layer(S.w1, x0, x1, kk, t, h);
+      unsigned a[3][4];
+      split_fragment(h, a);
+      const int col = kk * 16 + 2 * t;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        *reinterpret_cast<unsigned*>(&S.h1[k][row0][col]) = a[k][0];
+        *reinterpret_cast<unsigned*>(&S.h1[k][row1][col]) = a[k][1];
+        *reinterpret_cast<unsigned*>(&S.h1[k][row0][col + 8]) = a[k][2];
+        *reinterpret_cast<unsigned*>(&S.h1[k][row1][col + 8]) = a[k][3];
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) f1[kk][r][q] = fmaf(-h[r][q], h[r][q], 1.0f);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const unsigned b0 = *reinterpret_cast<const unsigned*>(&S.w2[j * 8 + g][col]);
+        const unsigned b1 = *reinterpret_cast<const unsigned*>(&S.w2[j * 8 + g][col + 8]);
+        mma_split(acc[j], low[j], a, b0, b1);
+      }
+    }
+    float y0 = 0.0f, y1 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int u = j * 8 + 2 * t + q;
+        const float w3 = S.wo[kW3 - kB2 + u], b2 = S.wo[u];
+        acc[j][q] = tanhf((acc[j][q] + low[j][q]) + b2);
+        acc[j][2 + q] = tanhf((acc[j][2 + q] + low[j][2 + q]) + b2);
+        y0 = fmaf(w3, acc[j][q], y0);
+        y1 = fmaf(w3, acc[j][2 + q], y1);
+      }
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 2);
+    // error, output-layer gradients, dz2 (in place of the activations)
+    const float b3 = S.wo[kB3 - kB2];
+    const float e0 = s0 < n ? y0 + b3 - target[s0] : 0.0f, e1 = s1 < n ? y1 + b3 - target[s1] : 0.0f;
+    const float dy0 = 2.0f * e0 * inv_n, dy1 = 2.0f * e1 * inv_n;
+    if (t == 0) {
+      lacc = fmaf(e0 * e0, inv_n, fmaf(e1 * e1, inv_n, lacc));
+      gb3 += dy0 + dy1;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float w3 = S.wo[kW3 - kB2 + j * 8 + 2 * t + q];
+        const float h0 = acc[j][q], h1 = acc[j][2 + q];
+        gw3[j][q] = fmaf(dy0, h0, fmaf(dy1, h1, gw3[j][q]));
+        acc[j][q] = dy0 * w3 * fmaf(-h0, h0, 1.0f);
+        acc[j][2 + q] = dy1 * w3 * fmaf(-h1, h1, 1.0f);
+        gb2[j][q] += acc[j][q] + acc[j][2 + q];
+      }
+    // backward through W2
+    float dh[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dh[j][q] = low[j][q] = 0.0f;
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const float v[2][4] = {{acc[2 * kk][0], acc[2 * kk][1], acc[2 * kk + 1][0], acc[2 * kk + 1][1]},
+                             {acc[2 * kk][2], acc[2 * kk][3], acc[2 * kk + 1][2], acc[2 * kk + 1][3]}};
+      unsigned a[3][4];
+      split_fragment(v, a);
+      const int col = kk * 16 + 2 * t;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        *reinterpret_cast<unsigned*>(&S.d2[k][row0][col]) = a[k][0];
+        *reinterpret_cast<unsigned*>(&S.d2[k][row1][col]) = a[k][1];
+        *reinterpret_cast<unsigned*>(&S.d2[k][row0][col + 8]) = a[k][2];
+        *reinterpret_cast<unsigned*>(&S.d2[k][row1][col + 8]) = a[k][3];
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const unsigned b0 = *reinterpret_cast<const unsigned*>(&S.w2t[j * 8 + g][col]);
+        const unsigned b1 = *reinterpret_cast<const unsigned*>(&S.w2t[j * 8 + g][col + 8]);
+        mma_split(dh[j], low[j], a, b0, b1);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int u = j * 8 + 2 * t + q, f = (j & 1) * 2 + q;
+        S.z1[row0][u] = (dh[j][q] + low[j][q]) * f1[j >> 1][0][f];
+        S.z1[row1][u] = (dh[j][2 + q] + low[j][2 + q]) * f1[j >> 1][1][f];
+      }
+    __syncthreads();
+    // dW2 += dz2^T h1 over the chunk's samples: the chunk's sum, then into gw2
+    float cw2[4][4], lw2[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cw2[i][q] = lw2[i][q] = 0.0f;
+#pragma unroll 2
+    for (int k0 = 0; k0 < kSamples; k0 += 16) {
+      const int r = lane & 7, m = lane >> 3;
+      unsigned a[3][4];
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        ldmatrix_trans(a[k], &S.d2[k][k0 + (m >> 1) * 8 + r][m0 + (m & 1) * 8]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        unsigned b[3][4];
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          ldmatrix_trans(b[k], &S.h1[k][k0 + (m & 1) * 8 + r][i0 + h * 16 + (m >> 1) * 8]);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          float(&l)[4] = lw2[h * 2 + s];
+          mma_bf16(l, a[2], b[0][2 * s], b[0][2 * s + 1]);
+          mma_bf16(l, a[0], b[2][2 * s], b[2][2 * s + 1]);
+          mma_bf16(l, a[1], b[1][2 * s], b[1][2 * s + 1]);
+          mma_bf16(l, a[1], b[0][2 * s], b[0][2 * s + 1]);
+          mma_bf16(l, a[0], b[1][2 * s], b[1][2 * s + 1]);
+          mma_add(cw2[h * 2 + s], a[0], b[0][2 * s], b[0][2 * s + 1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) gw2[i][q] += cw2[i][q] + lw2[i][q];
+    // dW1, db1: unit tid % 64, a quarter of the samples; the chunk's sum in two halves
+    {
+      const int u = tid & 63, q0 = (tid >> 6) * (kSamples / 4);
+      float part[2][5] = {};
+#pragma unroll 4
+      for (int q = q0; q < q0 + kSamples / 4; q += 2) {
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+          const float z = S.z1[q + o][u];
+          const float4 xv = *reinterpret_cast<const float4*>(S.x[q + o]);
+          part[o][0] = fmaf(z, xv.x, part[o][0]);
+          part[o][1] = fmaf(z, xv.y, part[o][1]);
+          part[o][2] = fmaf(z, xv.z, part[o][2]);
+          part[o][3] = fmaf(z, xv.w, part[o][3]);
+          part[o][4] += z;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 5; ++i) gw1[i] += part[0][i] + part[1][i];
+    }
+    __syncthreads();
+  }
+
+  // sums of the block into the gradient
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      atomicAdd(&grad[kW2 + (m0 + g + (q >> 1) * 8) * 64 + i0 + h * 8 + 2 * t + (q & 1)], gw2[h][q]);
+  // (one addition per block and parameter: more of them would add their rounding errors)
+  float* red = &S.z1[0][0];  // [warp][128 + 2]: db2 | dw3 | db3, loss
+  float* red1 = red + kGradThreads / 32 * 130;  // [quarter][dW1 | db1]
+  {
+    const int u = tid & 63, o = (tid >> 6) * 320;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) red1[o + u * 4 + i] = gw1[i];
+    red1[o + 256 + u] = gw1[4];
+  }
+  // over the rows g of a warp by shuffles, over the warps by shared memory
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float vb = gb2[j][q], vw = gw3[j][q];
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        vb += __shfl_xor_sync(0xffffffffu, vb, o);
+        vw += __shfl_xor_sync(0xffffffffu, vw, o);
+      }
+      if (g == 0) {
+        red[warp * 130 + j * 8 + 2 * t + q] = vb;
+        red[warp * 130 + 64 + j * 8 + 2 * t + q] = vw;
+      }
+    }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+    lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
+  }
+  if (lane == 0) {
+    red[warp * 130 + 128] = gb3;
+    red[warp * 130 + 129] = lacc;
+  }
+  __syncthreads();
+  for (int i = tid; i < 320; i += kGradThreads)  // W1 | b1
+    atomicAdd(&grad[kW1 + i], (red1[i] + red1[320 + i]) + (red1[640 + i] + red1[960 + i]));
+  if (tid < 130) {
+    float v = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kGradThreads / 32; ++w) v += red[w * 130 + tid];
+    // b2 | w3 | b3 follow one another in the parameters
+    atomicAdd(tid < 129 ? &grad[kB2 + tid] : loss, v);
+  }
+}
+
+// ---- inference -------------------------------------------------------------------------
 constexpr int kInferWarps = 4;
 
 __global__ void __launch_bounds__(32 * kInferWarps)
@@ -202,26 +428,10 @@ mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict
       for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-      // first-layer activations of this k-block: columns c0, c0+1 and c0+8, c0+9 of rows r0, r1
-      const int c0 = kk * 16 + 2 * t;
-      float h[2][4];  // [row][col c0, c0+1, c0+8, c0+9]
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int c = c0 + (q & 1) + (q >> 1) * 8;
-        float z0 = Wf[kB1 + c], z1 = Wf[kB1 + c];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          z0 = fmaf(Wf[kW1 + c * 4 + i], x0[i], z0);
-          z1 = fmaf(Wf[kW1 + c * 4 + i], x1[i], z1);
-        }
-        h[0][q] = tanhf(z0);
-        h[1][q] = tanhf(z1);
-      }
+      float h[2][4];
+      first_layer(Wf, x0, x1, kk, t, h);
       unsigned a[3][4];
-      split3(h[0][0], h[0][1], a[0][0], a[1][0], a[2][0]);
-      split3(h[1][0], h[1][1], a[0][1], a[1][1], a[2][1]);
-      split3(h[0][2], h[0][3], a[0][2], a[1][2], a[2][2]);
-      split3(h[1][2], h[1][3], a[0][3], a[1][3], a[2][3]);
+      split_fragment(h, a);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int nrow = j * 8 + g;  // output unit of this lane's B column
@@ -312,15 +522,17 @@ adg_status adg_mlp_grad(const uint16_t* params_bf16, const float* x, const float
   if (n == 0) return ADG_OK;
   if (n >= ((int64_t)1 << 31)) return mfail(ADG_ERR_INVALID, "too many samples");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  const size_t smem = sizeof(float) * kSmemFloats;
+  const size_t smem = sizeof(GradSmem);
   cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return mfail(ADG_ERR_CUDA, cudaGetErrorString(e));
   const int chunks = (int)((n + kSamples - 1) / kSamples);
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = chunks < sms ? chunks : sms;
-  mlp_grad_kernel<<<grid, kSamples, smem, s>>>(params_bf16, x, target, (int)n, 1.0f / (float)n, grad, loss);
+  // blocks of equal numbers of chunks: as few as need the same number of rounds (every block
+  // adds its sums to the gradient once, with its rounding)
+  const int rounds = (chunks + sms - 1) / sms, grid = (chunks + rounds - 1) / rounds;
+  mlp_grad_kernel<<<grid, kGradThreads, smem, s>>>(params_bf16, x, target, (int)n, 1.0f / (float)n, grad, loss);
   e = cudaGetLastError();
   return e == cudaSuccess ? ADG_OK : mfail(ADG_ERR_CUDA, cudaGetErrorString(e));
 }
