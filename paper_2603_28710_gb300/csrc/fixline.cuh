@@ -14,13 +14,13 @@
 //   * sum q v = 2^62 sum q1 f1 + 2^31 sum (q1 f0 + q0 f1) + sum q0 f0; the first two are exact
 //     in 64 bits (the host checks the bounds when it makes the tables); of the last only its
 //     mean 2^30 sum q0 is kept, as the start value of the second (with half a unit of the
-//     first for rounding);
+//     first for rounding; zeros start with the half unit alone, so that they give zeros);
 //   * the result is rounded to FP64 once.
 // Error before that rounding: typically 2^-59 of the largest value times the table's row sum.
 // An FP64 chain rounds once per term, each time by up to 2^-53 of its partial sum; emulated
 // on random lines its error is 4 to 10 times larger.
-// Values that hold Inf or NaN, or lie beyond the exponent range, go through the FP64 chain,
-// so non-finite values spread as they do there.
+// Values that hold Inf or NaN, or are too large or too small for the exponent range (about
+// 10^-290 to 10^303), go through the FP64 chain, so non-finite values spread as they do there.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -32,10 +32,14 @@ namespace adg {
 // Upper 31 bits of |x|: its magnitude as an ordered integer, its exponent field from bit 20.
 __device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7FFFFFFF; }
 
-// Exponent of the largest magnitude (abs_hi), clamped from below: smaller values are then
-// rounded at 2^-1020 of the clamp, below any result of a normal computation.
+// Exponent of the largest magnitude (abs_hi); zeros take the smallest one.
 __device__ __forceinline__ int fixed_exponent(const FixedScale& s, int max_hi) {
   return max(max_hi >> 20, s.elo);
+}
+// Whether the magnitude is outside of the range in which 60 bits below it and the results are
+// normal numbers (zero is inside): the values then go through the FP64 chain.
+__device__ __forceinline__ bool fixed_outside(const FixedScale& s, int max_hi) {
+  return (max_hi >> 20) > s.ehi || (unsigned)(max_hi - 1) < (unsigned)((s.elo << 20) - 1);
 }
 
 // (hi, lo) -> -(hi, lo) where the top bit of s is set
@@ -103,6 +107,12 @@ __device__ __forceinline__ double fixed_result(const FixedAcc& t, const FixedSca
   return fixed_to_double(t.a + (t.m >> 31), e + s.eout);
 }
 
+// Start value of the middle limb sum for values of exponent e.
+constexpr long long kFixedHalf = 1ll << 30;
+__device__ __forceinline__ long long fixed_start(const FixedScale& s, int e, long long c) {
+  return e > s.elo ? c : kFixedHalf;
+}
+
 // Traces at both ends of a line of N nodes (low end -1, high end +1).
 template <int N>
 __device__ __forceinline__ void line_traces(const FixedTrace& T, const OpTables* tab,
@@ -111,7 +121,7 @@ __device__ __forceinline__ void line_traces(const FixedTrace& T, const OpTables*
 #pragma unroll
   for (int a = 0; a < N; ++a) m = max(m, abs_hi(x[a]));
   const int e = fixed_exponent(T.s, m);
-  if (e > T.s.ehi) {
+  if (fixed_outside(T.s, m)) {
     lo = hi = 0.0;
 #pragma unroll
     for (int a = 0; a < N; ++a) {
@@ -128,7 +138,7 @@ __device__ __forceinline__ void line_traces(const FixedTrace& T, const OpTables*
   }
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
-    long long s = T.c[side];
+    long long s = fixed_start(T.s, e, T.c[side]);
 #pragma unroll
     for (int a = 0; a < N; ++a) {
       s = mad_wide(T.t[side][a].x, f[a].y, s);

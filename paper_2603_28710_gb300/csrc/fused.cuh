@@ -437,7 +437,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
             fex[v] = fixed_exponent(fsc, sMax[el * NV + v]);
-            chain = chain || fex[v] > fsc.ehi;
+            chain = chain || fixed_outside(fsc, sMax[el * NV + v]);
           }
 #pragma unroll
           for (int d = 0; d < D; ++d)
@@ -473,9 +473,10 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           FixedAcc fa[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) {
-            fa[v] = FixedAcc{0, 0};
+            long long c = 0;
 #pragma unroll
-            for (int d = 0; d < D; ++d) fa[v].m += ftab->c[d][ix[d]];
+            for (int d = 0; d < D; ++d) c += ftab->c[d][ix[d]];
+            fa[v] = FixedAcc{0, fixed_start(fsc, fex[v], c)};
           }
 #pragma unroll
           for (int d = 0; d < D; ++d) {

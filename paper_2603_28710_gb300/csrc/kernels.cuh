@@ -1011,8 +1011,9 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
   if (active) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      ex[v] = fixed_exponent(sc, sMax[el * NV + v]);
-      chain = chain || ex[v] > sc.ehi;
+      const int mx = sMax[el * NV + v];
+      ex[v] = fixed_exponent(sc, mx);
+      chain = chain || fixed_outside(sc, mx);
     }
     if (!chain) {
 #pragma unroll
@@ -1045,7 +1046,7 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
 #pragma unroll
       for (int d = 1; d < D; ++d) c += sC[d * N + ix[d]];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] = FixedAcc{0, c};
+      for (int v = 0; v < NV; ++v) acc[v] = FixedAcc{0, fixed_start(sc, ex[v], c)};
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
