@@ -86,8 +86,8 @@ typedef enum {
 } adg_precision;
 
 typedef enum {
-  ADG_PATH_AUTO = 0,   /* the faster path on GB300 for the arithmetic: ADG_PATH_ELEMENT
-                          for FP32, ADG_PATH_SPLIT for FP64 and FP32 pairs               */
+  ADG_PATH_AUTO = 0,   /* the faster path on GB300: for FP32 ADG_PATH_ELEMENT up to about
+                          10^6 nodes (degree 3: at every size), otherwise ADG_PATH_SPLIT  */
   ADG_PATH_SPLIT = 1,  /* per RK stage a face-flux launch, then a volume/update launch    */
   ADG_PATH_FUSED = 2,  /* per RK stage one launch per tile of elements: face fluxes and
                           volume/update work together, tiles staged by TMA copies        */

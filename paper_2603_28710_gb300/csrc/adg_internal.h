@@ -20,6 +20,7 @@ struct FixedTrace {  // rows l_a(-1) and l_a(+1), the limbs of an entry side by 
   int2 t[2][kMaxN];
   long long c[2];  // start values of the middle limb sums (fixline.cuh)
   FixedScale s;
+  float2 w[2][kMaxN];  // the rows in FP32, each value twice (packed FP32 operator)
 };
 struct FixedSweep {  // direction d, row i: N flux weights, low-face and high-face weight
   int2 q[3][kMaxN * (kMaxN + 2)];  // entry [i*(N+2) + k]
@@ -56,6 +57,9 @@ struct OpTables {
   // the tables (unscaled and dt-scaled) and the trace weights in fixed point
   FixedSweep fx, fxs;
   FixedTrace ft;
+  // FP32 sweep tables of the packed FP32 operator: Qf and Qsf in FP32, each value twice
+  float2 qp[3][kMaxN * kMaxN];
+  float2 qps[3][kMaxN * kMaxN];
 };
 
 struct MeshArgs {
@@ -107,7 +111,9 @@ struct __align__(16) VolArgs {
   int scaled;            // 1: use the dt-scaled tables (2N), the accumulator is dt * k
   int bulk;              // 1: n_elem * nodes is a multiple of 4, so the element path may
                          // stage whole tiles by TMA bulk copies (16-byte aligned rows)
-  FixedTrace ft;         // trace weights (FP64 trace arithmetic)
+  FixedTrace ft;         // trace weights (FP64 and FP32 operators)
+  const OpTables* tab_host;  // the tables in host memory: launches of the FP32 operator pass
+                             // its sweep rows as a kernel argument
 };
 
 struct __align__(16) FluxArgs {
@@ -191,6 +197,18 @@ cudaError_t launch_samples(const double* log, int64_t rec_len, int stages, const
 cudaError_t launch_log_traces(int prec, int dim, int N, const void* tr, const int32_t* face_d,
                               const int32_t* face_e, const MeshArgs& m, int64_t npe, double* out,
                               cudaStream_t s);
+
+// ADG_PATH_AUTO: whether the element path is the faster one.  FP32 only (the FP64 operator would
+// evaluate every interior face twice on the pipe that bounds it, and so would the pairs).
+// FP32, GB300, us per stage element / split: one launch instead of two up to about 10^6 nodes
+// (35^2 p=4 3.2 / 4.5, 100^2 8.6 / 9.1, 141^2 12.9 / 13.7; 16^3 p=3 13.3 / 13.7); above, the
+// second evaluation of every interior face costs more than the launch and the flux array
+// (256^2 p=4 47.7 / 47.1, 640^2 p=1 60.0 / 56.6, 64^3 p=2 424 / 366, 40^3 p=4 382 / 342, 32^3
+// p=5 329 / 315), except with four nodes per direction, whose tiles fill their warps in every
+// phase (320^2 p=3 42.9 / 45.5, 48^3 289 / 288).
+inline bool element_path_faster(int prec, int N, int64_t nodes) {
+  return prec == 1 && (N == 4 || nodes < ((int64_t)1 << 20));
+}
 
 // Launchers (one per arithmetic), implemented in the kernel translation units.
 // prec: 0 = FP64, 1 = FP32, 2 = FP32 pair.

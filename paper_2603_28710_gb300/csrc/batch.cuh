@@ -75,11 +75,22 @@ template <int D, int N> struct VolRegs<D, N, float> {
   static constexpr int value = D != 2 ? 56 : ((N == 4 || N == 8) ? 48 : 40);
 };
 
+// Sweep table of the instance whose arguments `a` hold, into shared memory (FP32 operator).
+template <int D, int N>
+__device__ __forceinline__ void stage_tab(PackTab<D, N>* t, const VolArgs& a) {
+  const float2(&q)[3][kMaxN * kMaxN] = a.scaled ? a.tab->qps : a.tab->qp;
+  constexpr int Q = N * N;
+  for (int i = threadIdx.x; i < D * Q; i += blockDim.x) t->q[i / Q][i % Q] = q[i / Q][i % Q];
+}
+template <int D, int N>
+__device__ __forceinline__ void stage_tab(NoTab*, const VolArgs&) {}
+
 template <int D, int N, typename R, int TT>
-__global__ void __launch_bounds__(Tile<D, N, TT>::THREADS,
-                                  min_blocks_for(VolRegs<D, N, R>::value, Tile<D, N, TT>::THREADS))
+__global__ void __launch_bounds__(vol_block<R>(Tile<D, N, TT>::THREADS),
+                                  min_blocks_for(VolRegs<D, N, R>::value, vol_block<R>(Tile<D, N, TT>::THREADS)))
 batch_vol_kernel(const VolArgs* va, int nstages, int stage, BatchGroupArgs g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) SweepArg<D, N, R> st;
   __shared__ __align__(16) VolArgs sa;
   __shared__ int soff[kMaxSharedOffsets];
   const int* off = stage_offsets(g, soff);
@@ -89,9 +100,11 @@ batch_vol_kernel(const VolArgs* va, int nstages, int stage, BatchGroupArgs g) {
     if (k != cur) {
       stage_args(&sa, &va[g.inst[k] * nstages + stage]);
       __syncthreads();
+      stage_tab<D, N>(&st, sa);
+      __syncthreads();
       cur = k;
     }
-    vol_body<D, N, R, TT>(sa, vb - off[k], smem_raw);
+    vol_body<D, N, R, TT>(sa, st, vb - off[k], smem_raw);
     __syncthreads();  // shared memory (and sa) are reused by the next virtual block
   }
 }
@@ -124,12 +137,13 @@ batch_vol_kernel_fp64(const VolArgs* va, int nstages, int stage, BatchGroupArgs 
 template <int D, int N, typename R> struct VolFacesBatchRegs { static constexpr int value = D == 2 ? 72 : 80; };
 
 template <int D, int N, typename R, int TT>
-__global__ void __launch_bounds__(Tile<D, N, TT>::THREADS,
+__global__ void __launch_bounds__(vol_block<R>(Tile<D, N, TT>::THREADS),
                                   min_blocks_for(VolFacesBatchRegs<D, N, R>::value,
-                                                 Tile<D, N, TT>::THREADS))
+                                                 vol_block<R>(Tile<D, N, TT>::THREADS)))
 batch_vol_faces_kernel(const VolArgs* va, const FluxArgs* fa, int nstages, int stage,
                        BatchGroupArgs g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) SweepArg<D, N, R> st;
   __shared__ __align__(16) VolArgs sa;
   __shared__ __align__(16) FluxArgs sf;
   __shared__ int soff[kMaxSharedOffsets];
@@ -141,9 +155,11 @@ batch_vol_faces_kernel(const VolArgs* va, const FluxArgs* fa, int nstages, int s
       stage_args(&sa, &va[g.inst[k] * nstages + stage]);
       stage_args(&sf, &fa[g.inst[k] * nstages + stage]);
       __syncthreads();
+      stage_tab<D, N>(&st, sa);
+      __syncthreads();
       cur = k;
     }
-    vol_body<D, N, R, TT, false, ElementFaces>(sa, vb - off[k], smem_raw, ElementFaces{sf, sf.tr});
+    vol_body<D, N, R, TT, false, ElementFaces>(sa, st, vb - off[k], smem_raw, ElementFaces{sf, sf.tr});
     __syncthreads();  // shared memory (and the arguments) are reused by the next virtual block
   }
 }
@@ -184,7 +200,7 @@ struct BatchDispatch {
       return go(batch_vol_kernel_fp64<D, N, TT>, VolSmem64<D, N, TT>::BLOCK, VolSmem64<D, N, TT>::BYTES, va, ns,
                 st, g, grid, s, occ);
     } else {
-      return go(batch_vol_kernel<D, N, R, TT>, T::THREADS, vol_flux_bytes<D, N, R, TT>(), va, ns, st, g,
+      return go(batch_vol_kernel<D, N, R, TT>, vol_block<R>(T::THREADS), vol_flux_bytes<D, N, R, TT>(), va, ns, st, g,
                 grid, s, occ);
     }
   }
@@ -209,8 +225,8 @@ struct BatchDispatch {
     }
     if (occ)
       return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_vol_faces_kernel<D, N, R, TT>,
-                                                           T::THREADS, smem);
-    batch_vol_faces_kernel<D, N, R, TT><<<grid, T::THREADS, smem, s>>>(va, fa, ns, st, g);
+                                                           vol_block<R>(T::THREADS), smem);
+    batch_vol_faces_kernel<D, N, R, TT><<<grid, vol_block<R>(T::THREADS), smem, s>>>(va, fa, ns, st, g);
     return cudaGetLastError();
   }
   template <int D, int N>

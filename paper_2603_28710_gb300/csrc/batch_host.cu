@@ -382,6 +382,10 @@ adg_status adg_batch_create(int n, const adg_mesh* meshes, const int* degrees, c
   // as separate handles take the split or element path (both give the split path's bits),
   // so results equal separate split-path handles bit for bit
   if (o.kernel_path == ADG_PATH_FUSED) o.kernel_path = ADG_PATH_SPLIT;
+  // (the graph's FP32 launches take the element path at every size, so every handle gets its
+  // second trace buffer; the choice for separate stepping is made below)
+  const bool automatic = o.kernel_path == ADG_PATH_AUTO && o.precision == ADG_PREC_FP32;
+  if (automatic) o.kernel_path = ADG_PATH_ELEMENT;
   adg_batch* b = new (std::nothrow) adg_batch();
   if (!b) return bfail(nullptr, ADG_ERR_OOM, "host allocation failed");
   b->n = n;
@@ -402,6 +406,7 @@ adg_status adg_batch_create(int n, const adg_mesh* meshes, const int* degrees, c
       delete b;
       return bfail(nullptr, st, msg);
     }
+    if (automatic) s->faces = element_path_faster(s->prec, s->N, s->ne * s->ND);
     b->inst.push_back(s);
   }
   b->stages = b->inst[0]->stages;

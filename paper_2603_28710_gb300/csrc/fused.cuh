@@ -360,7 +360,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           elow = elem_shift(m, eh, ec, d, -1);
 #pragma unroll
           for (int v = 0; v < NV; ++v)
-            wm[v] = Arith<R>::load(trg + (((d * 2 + 1) * NV + v) * ne + elow) * NF + j);
+            wm[v] = Arith<R>::load(trg + TraceLay<D, N, R>::at(ne, d * 2 + 1, v, elow, j));
         }
         if (c < Ed) {
           const int te = (zh * TY + yh) * TX + xh;
@@ -373,7 +373,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           const int ehi = elem_shift(m, el_, ec, d, +1);
 #pragma unroll
           for (int v = 0; v < NV; ++v)
-            wp[v] = Arith<R>::load(trg + (((d * 2 + 0) * NV + v) * ne + ehi) * NF + j);
+            wp[v] = Arith<R>::load(trg + TraceLay<D, N, R>::at(ne, d * 2, v, ehi, j));
         }
         const int slot = A.f.pe_mode ? A.f.pe_slot[d * ne + elow] : -1;
         face_flux<D, N, R>(A.f, d, slot, j, wm, wp, c >= 1, fl);
@@ -657,7 +657,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
           val = interp_line<N, C>(t, src, stride);
         }
-        store_trace(tro + (((d * 2 + side) * NV + v) * ne + gel(x, y, z)) * NF + j, val);
+        store_trace(tro + TraceLay<D, N, R>::at(ne, d * 2 + side, v, gel(x, y, z), j), val);
       }
     }
     __syncthreads();  // the slot and BIG are free for the next tile

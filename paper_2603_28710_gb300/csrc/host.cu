@@ -191,6 +191,11 @@ void fixed_sweep_tables(const adg_solver* s, double dt, bool scaled, FixedSweep*
   f->s = fixed_scale(67 - (scaled ? s->fix_s + 53 - sh - ex : s->fix_s - sh));
 }
 
+// packed FP32 sweep table from the FP32-pair one
+void packed_table(int N, const float2* Q, float2* out) {
+  for (int i = 0; i < N * N; ++i) out[i] = make_float2(Q[i].x, Q[i].x);
+}
+
 void build_tables(adg_solver* s) {
   const int N = s->N;
   OpTables& T = s->tab;
@@ -264,7 +269,10 @@ void build_tables(adg_solver* s) {
     for (int a = 0; a < N; ++a) {
       T.ft.t[0][a] = fixed_entry((int64_t)llroundl(ldexpl(lm[a], st)));
       T.ft.t[1][a] = fixed_entry((int64_t)llroundl(ldexpl(lp[a], st)));
+      T.ft.w[0][a] = make_float2(T.Tmf[a].x, T.Tmf[a].x);
+      T.ft.w[1][a] = make_float2(T.Tpf[a].x, T.Tpf[a].x);
     }
+    for (int d = 0; d < s->dim; ++d) packed_table(N, T.Qf[d], T.qp[d]);
     for (int side = 0; side < 2; ++side) {
       T.ft.c[side] = (long long)1 << 30;
       for (int a = 0; a < N; ++a) T.ft.c[side] += T.ft.t[side][a].y / 2;
@@ -612,6 +620,8 @@ adg_status upload_dt_tables(adg_solver* s) {
     }
   }
   fixed_sweep_tables(s, s->dt, true, &s->tab.fxs);
+  for (int d = 0; d < s->dim; ++d)
+    packed_table(s->N, s->tab.Qsf[d], s->tab.qps[d]);
   ADG_CUDA(s, cudaMemcpyAsync(s->tab_dev, &s->tab, sizeof(OpTables), cudaMemcpyHostToDevice, s->stream));
   return ADG_OK;
 }
@@ -665,6 +675,22 @@ CkptHeader ckpt_header(const adg_solver* s) {
   h.dt = s->dt;
   h.gamma = s->opt.gamma;
   return h;
+}
+
+// Checkpoints hold the traces as [d][side][v][e][j]; the FP32 operator keeps them on the device
+// as [d][side][e][j][v] (kernels.cuh, TraceLay).  In-place conversion of a host copy.
+void ckpt_traces_convert(const adg_solver* s, unsigned char* p, bool to_file) {
+  if (s->prec != 1) return;
+  const int64_t rows = s->ne * s->NF;
+  std::vector<float> t((size_t)(rows * s->NV));
+  for (int ds = 0; ds < 2 * s->dim; ++ds, p += sizeof(float) * t.size()) {
+    std::memcpy(t.data(), p, sizeof(float) * t.size());
+    for (int64_t r = 0; r < rows; ++r)
+      for (int v = 0; v < s->NV; ++v) {
+        const int64_t file = v * rows + r, dev = r * s->NV + v;
+        std::memcpy(p + 4 * (to_file ? file : dev), &t[(size_t)(to_file ? dev : file)], 4);
+      }
+  }
 }
 
 int64_t ckpt_bytes(const adg_solver* s) {
@@ -733,6 +759,7 @@ VolArgs stage_vol_args(const adg_solver* s, int m) {
   va.scaled = s->rk2n ? 1 : 0;
   va.bulk = (s->ne * s->ND) % 4 == 0 ? 1 : 0;
   va.ft = s->tab.ft;
+  va.tab_host = &s->tab;
   return va;
 }
 
@@ -855,13 +882,10 @@ adg_status adg_create(const adg_mesh* mesh, int degree, const int P[3], int max_
   // between the two launches)
   s->fused = flux != ADG_FLUX_LEARNED && fused_tile(s->dim, s->N, s->tile) &&
              o.kernel_path == ADG_PATH_FUSED;
-  // element path on request, and by default for the FP32 operator: it evaluates every
-  // interior face twice, which the FP32 form (bound by memory and issue) affords and the
-  // FP64 and pair forms (bound by the FP64 pipe) do not (measured on GB300: FP32 +2 to
-  // +6 %, FP64 -24 %, pairs -21 % in 2D and -46 % in 3D)
+  // element path on request, and by default where it is the faster one
   s->faces = flux != ADG_FLUX_LEARNED &&
              (o.kernel_path == ADG_PATH_ELEMENT ||
-              (o.kernel_path == ADG_PATH_AUTO && o.precision == ADG_PREC_FP32));
+              (o.kernel_path == ADG_PATH_AUTO && element_path_faster(s->prec, s->N, ne * s->ND)));
   for (int d = 0; d < 3; ++d) {
     if (d >= s->dim) s->tile[d] = 1;
     s->ntile[d] = (s->margs.n[d] + s->tile[d] - 1) / s->tile[d];
@@ -1186,11 +1210,17 @@ adg_status adg_checkpoint_save(adg_solver* s, void* buf, int64_t bytes) {
   const size_t sb = prec_bytes(s->prec);
   ADG_CUDA(s, cudaMemcpyAsync(p, s->w, (size_t)h.ndof * 8, cudaMemcpyDeviceToHost, s->stream));
   p += (size_t)h.ndof * 8;
+  unsigned char* traces = p;
   ADG_CUDA(s, cudaMemcpyAsync(p, s->tr, (size_t)h.n_tr * sb, cudaMemcpyDeviceToHost, s->stream));
   p += (size_t)h.n_tr * sb;
   if (h.n_ring > 0)
     ADG_CUDA(s, cudaMemcpyAsync(p, s->ring, (size_t)h.n_ring * sb, cudaMemcpyDeviceToHost, s->stream));
   ADG_CUDA(s, cudaStreamSynchronize(s->stream));
+  try {
+    ckpt_traces_convert(s, traces, true);
+  } catch (const std::bad_alloc&) {
+    return fail(s, ADG_ERR_OOM, "host allocation failed");
+  }
   return ADG_OK;
 }
 
@@ -1223,7 +1253,18 @@ adg_status adg_checkpoint_restore(adg_solver* s, const void* buf, int64_t bytes)
   const size_t sb = prec_bytes(s->prec);
   ADG_CUDA(s, cudaMemcpyAsync(s->w, p, (size_t)h.ndof * 8, cudaMemcpyHostToDevice, s->stream));
   p += (size_t)h.ndof * 8;
-  ADG_CUDA(s, cudaMemcpyAsync(s->tr, p, (size_t)h.n_tr * sb, cudaMemcpyHostToDevice, s->stream));
+  std::vector<unsigned char> traces;  // a copy in the device's order (FP32)
+  const unsigned char* tr_src = p;
+  if (s->prec == 1) {
+    try {
+      traces.assign(p, p + (size_t)h.n_tr * sb);
+      ckpt_traces_convert(s, traces.data(), false);
+    } catch (const std::bad_alloc&) {
+      return fail(s, ADG_ERR_OOM, "host allocation failed");
+    }
+    tr_src = traces.data();
+  }
+  ADG_CUDA(s, cudaMemcpyAsync(s->tr, tr_src, (size_t)h.n_tr * sb, cudaMemcpyHostToDevice, s->stream));
   p += (size_t)h.n_tr * sb;
   if (h.n_ring > 0)
     ADG_CUDA(s, cudaMemcpyAsync(s->ring, p, (size_t)h.n_ring * sb, cudaMemcpyHostToDevice, s->stream));
@@ -1272,6 +1313,7 @@ adg_status adg_rhs(adg_solver* s, const double* u, double* k, int64_t count, int
   va.fl = s->fl;
   va.tr = s->tr;
   va.write_traces = 0;
+  va.tab_host = &s->tab;
   ADG_CUDA(s, launch_vol(s->prec, s->dim, s->N, va, s->stream));
   if (!on_device)
     ADG_CUDA(s, cudaMemcpyAsync(k, s->tmp_k, bytes, cudaMemcpyDeviceToHost, s->stream));

@@ -42,25 +42,6 @@ struct Tile {
   static constexpr int THREADS = EPB * ND;
 };
 
-// Element strides (in values) of the volume kernel's shared-memory tiles.  For 4-byte
-// values the stride is padded to be congruent to the node count modulo the 32 banks, so
-// that a warp's consecutive nodes fall into consecutive banks across element boundaries
-// (unpadded, a 2D p=4 FP32 tile put two elements' nodes into the same banks: 2-way
-// conflicts on every store of the pointwise fluxes and the next stage input).
-constexpr int bank_pad(int base, int nd, int bytes) {
-  return bytes == 4 ? ((nd - base) % 32 + 32) % 32 : 0;
-}
-template <int D, int N, typename R>
-constexpr int sf_stride() {  // pointwise fluxes [el][D][NV][ND]
-  return D * (D + 2) * IPow<N, D>::value +
-         bank_pad(D * (D + 2) * IPow<N, D>::value, IPow<N, D>::value, (int)sizeof(R));
-}
-template <int D, int N, typename C>
-constexpr int sx_stride() {  // next stage input [el][NV][ND]
-  return (D + 2) * IPow<N, D>::value +
-         bank_pad((D + 2) * IPow<N, D>::value, IPow<N, D>::value, (int)sizeof(C));
-}
-
 // floor(e / m.n[i]) for 0 <= e < 2^31 (multiply-high by the precomputed inverse)
 __device__ __forceinline__ int mesh_div(const MeshArgs& m, int i, int e) {
   return m.n[i] == 1 ? e : (int)(__umulhi((unsigned)e, m.divm[i]) >> m.divs[i]);
@@ -322,6 +303,199 @@ __device__ __forceinline__ void store_trace(float2* p, double v) {
 }
 __device__ __forceinline__ void store_trace(float2* p, df64 v) { *p = make_float2(v.hi, v.lo); }
 
+// Layout of the trace arrays: [d][side][v][e][j], in the FP32 operator [d][side][e][j][v] -- the
+// variables of a face node together, so that a 2D node's traces are one 16-byte access (in 3D
+// five accesses from one address).
+template <int D, int N, typename R>
+struct TraceLay {
+  static constexpr int NF = IPow<N, D - 1>::value, NV = D + 2;
+  static constexpr bool kTogether = std::is_same<R, float>::value;
+  // ds = 2 d + side (side 1: the element's +d face)
+  __device__ static __forceinline__ int at(int ne, int ds, int v, int e, int j) {
+    return kTogether ? ((ds * ne + e) * NF + j) * NV + v : ((ds * NV + v) * ne + e) * NF + j;
+  }
+};
+
+// Layout of the face-flux array: [d][v][e][j], in the FP32 operator [d][e][j][v].
+template <int D, int N, typename R>
+struct FluxLay {
+  static constexpr int NF = IPow<N, D - 1>::value, NV = D + 2;
+  __device__ static __forceinline__ int at(int ne, int d, int v, int e, int j) {
+    return TraceLay<D, N, R>::kTogether ? ((d * ne + e) * NF + j) * NV + v : ((d * NV + v) * ne + e) * NF + j;
+  }
+};
+
+// The traces of one face node.
+template <int D, int N, typename R>
+__device__ __forceinline__ void load_traces(const typename Arith<R>::S* tr, int ne, int ds, int e, int j,
+                                            R (&w)[D + 2]) {
+  using Lay = TraceLay<D, N, R>;
+  if constexpr (Lay::kTogether && D == 2) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(tr + Lay::at(ne, ds, 0, e, j)));
+    w[0] = q.x;
+    w[1] = q.y;
+    w[2] = q.z;
+    w[3] = q.w;
+  } else if constexpr (Lay::kTogether) {
+    const float* q = tr + Lay::at(ne, ds, 0, e, j);
+#pragma unroll
+    for (int v = 0; v < D + 2; ++v) w[v] = __ldg(q + v);
+  } else {
+#pragma unroll
+    for (int v = 0; v < D + 2; ++v) w[v] = Arith<R>::load(tr + Lay::at(ne, ds, v, e, j));
+  }
+}
+
+// The fluxes of one face node (FP32 operator).
+template <int D, int N>
+__device__ __forceinline__ void load_flux(const float* fl, int ne, int d, int e, int j, float (&f)[D + 2]) {
+  const float* p = fl + FluxLay<D, N, float>::at(ne, d, 0, e, j);
+  if constexpr (D == 2) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    f[0] = q.x;
+    f[1] = q.y;
+    f[2] = q.z;
+    f[3] = q.w;
+  } else {
+#pragma unroll
+    for (int v = 0; v < D + 2; ++v) f[v] = __ldg(p + v);
+  }
+}
+
+// Shared-memory array of the values of all variables at a node in the FP32 operator: four as
+// one float4, the fifth (3D) in an array of its own behind the CNT float4.
+template <int D, int CNT>
+struct NodeArray {
+  static constexpr size_t BYTES = (CNT * (sizeof(float4) + (D == 3 ? sizeof(float) : 0)) + 15) / 16 * 16;
+  float4* a;
+  __device__ explicit NodeArray(unsigned char* p) : a(reinterpret_cast<float4*>(p)) {}
+  __device__ __forceinline__ float* b() const { return reinterpret_cast<float*>(a + CNT); }
+  __device__ __forceinline__ void store(int i, const float (&f)[D + 2]) const {
+    a[i] = make_float4(f[0], f[1], f[2], f[3]);
+    if constexpr (D == 3) b()[i] = f[4];
+  }
+  // variables 2 pair and 2 pair + 1 of node i
+  __device__ __forceinline__ float2& pair(int i, int p) const { return reinterpret_cast<float2*>(a)[2 * i + p]; }
+  __device__ __forceinline__ void load(int i, float (&f)[D + 2]) const {
+    const float4 q = a[i];
+    f[0] = q.x;
+    f[1] = q.y;
+    f[2] = q.z;
+    f[3] = q.w;
+    if constexpr (D == 3) f[4] = b()[i];
+  }
+};
+
+// A NodeArray over the nodes of a tile: x-lines of 4 or 8 nodes are padded by one value, so that
+// the lines that the lanes of a warp read start in different banks (unpadded a warp's access
+// along x takes 4 or 8 passes: 160^2 p=7 48 against 40 us; 2 and 6 nodes take 2 passes, and
+// padding them costs more in occupancy: 96^3 p=1 418 against 398 us).
+template <int D, int N, int TT>
+struct TileNodes : NodeArray<D, Tile<D, N, TT>::THREADS / N * (N + (N % 4 == 0 ? 1 : 0))> {
+  static constexpr int PN = N + (N % 4 == 0 ? 1 : 0);
+  using NodeArray<D, Tile<D, N, TT>::THREADS / N * PN>::NodeArray;
+  __device__ static __forceinline__ int at(int node) { return node + (PN - N) * (node / N); }
+};
+
+// Sweep table of the FP32 operator as a kernel argument (each weight twice, for packed
+// instructions): entries have compile-time addresses in the constant bank.  The other
+// operators read theirs from memory.
+template <int D, int N>
+struct PackTab {
+  float2 q[D][N * N];
+};
+struct NoTab {};
+template <int D, int N, typename R>
+using SweepArg = std::conditional_t<std::is_same<R, float>::value, PackTab<D, N>, NoTab>;
+template <int D, int N, typename R>
+SweepArg<D, N, R> sweep_arg(const VolArgs& a) {
+  SweepArg<D, N, R> t;
+  if constexpr (std::is_same<R, float>::value) {
+    for (int d = 0; d < D; ++d)
+      for (int i = 0; i < N * N; ++i) t.q[d][i] = (a.scaled ? a.tab_host->qps : a.tab_host->qp)[d][i];
+  }
+  return t;
+}
+
+// Threads of a volume-kernel block: the FP32 form's line phases stride by whole warps.
+template <typename R>
+constexpr int vol_block(int threads) {
+  return std::is_same<R, float>::value ? (threads + 31) / 32 * 32 : threads;
+}
+
+// First value and stride of line r (= el * NF + j) along d of a tile of elements whose x-lines
+// take PN values each (PN = N: the nodes as they are; PN > N: padded).
+template <int D, int N, int PN>
+__device__ __forceinline__ int tile_line(int d, int r, int& st) {
+  constexpr int NF = IPow<N, D - 1>::value, NDP = PN * NF;
+  st = 1;
+  if (d == 0) return r * PN;
+  const int el = r / NF, j = r - el * NF;
+  const int base = el * NDP + j;
+  st = PN;
+  if constexpr (D == 3) {
+    const int c = j / N;  // j = (a, c): z for d = 1, y for d = 2
+    if (d == 1) return base + c * (PN * N - N);
+    st = PN * N;
+    return base + c * (PN - N);
+  } else {
+    return base;
+  }
+}
+
+// FP32 traces of a tile of elements (node i of the tile in x) -> tr: one thread per (direction,
+// line) interpolates all variables at both ends of its line, two variables per instruction.
+template <int D, int N, int TT>
+__device__ __forceinline__ void write_traces_fp32(const MeshArgs& m, const FixedTrace& ft,
+                                                  const TileNodes<D, N, TT>& x, int e0,
+                                                  float* tr) {
+  using T = Tile<D, N, TT>;
+  using Nodes = TileNodes<D, N, TT>;
+  using Lay = TraceLay<D, N, float>;
+  constexpr int NF = T::NF, NV = T::NV, LINES = T::EPB * NF;
+  const int ne = (int)m.ne;
+  const int last = (ne - e0) * NF;  // lines of the tile's elements inside the mesh
+  for (int g = threadIdx.x; g < D * LINES; g += blockDim.x) {
+    const int d = g / LINES, r = g - d * LINES;  // r = el * NF + j
+    if (r >= last) continue;
+    int st;
+    const int base = tile_line<D, N, Nodes::PN>(d, r, st);
+    float2 lo[D], hi[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) lo[i] = hi[i] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      const float4 q = x.a[base + a * st];
+      const float2 q0 = make_float2(q.x, q.y), q1 = make_float2(q.z, q.w);
+      lo[0] = __ffma2_rn(ft.w[0][a], q0, lo[0]);
+      lo[1] = __ffma2_rn(ft.w[0][a], q1, lo[1]);
+      hi[0] = __ffma2_rn(ft.w[1][a], q0, hi[0]);
+      hi[1] = __ffma2_rn(ft.w[1][a], q1, hi[1]);
+      if constexpr (D == 3) {
+        const float f = x.b()[base + a * st];
+        lo[2].x = fmaf(ft.w[0][a].x, f, lo[2].x);
+        hi[2].x = fmaf(ft.w[1][a].x, f, hi[2].x);
+      }
+    }
+    float* dst = tr + Lay::at(ne, 2 * d, 0, e0, 0) + r * NV;
+    const int side = ne * NF * NV;
+    if constexpr (D == 2) {
+      *reinterpret_cast<float4*>(dst) = make_float4(lo[0].x, lo[0].y, lo[1].x, lo[1].y);
+      *reinterpret_cast<float4*>(dst + side) = make_float4(hi[0].x, hi[0].y, hi[1].x, hi[1].y);
+    } else {
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const float2(&f)[D] = o ? hi : lo;
+        dst[o * side] = f[0].x;
+        dst[o * side + 1] = f[0].y;
+        dst[o * side + 2] = f[1].x;
+        dst[o * side + 3] = f[1].y;
+        dst[o * side + 4] = f[D - 1].x;
+      }
+    }
+  }
+}
+
 // FP64 traces of a tile of elements in shared memory (value (el, v, node) at v * VS + el * ND +
 // node) -> tr: one thread per (direction, variable, line) interpolates both ends of
 // its line in fixed point (fixline.cuh).
@@ -330,26 +504,15 @@ __device__ __forceinline__ void write_traces_fp64(const MeshArgs& m, const Fixed
                                                   const OpTables* tab, const double* sX, int VS,
                                                   int e0, double* tr) {
   using T = Tile<D, N, TT>;
-  constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB, LINES = EPB * NF;
+  constexpr int NF = T::NF, NV = T::NV, EPB = T::EPB, LINES = EPB * NF;
   const int ne = (int)m.ne;
   const int last = (ne - e0) * NF;  // lines of the tile's elements inside the mesh
   for (int g = threadIdx.x; g < D * NV * LINES; g += blockDim.x) {
     const int dv = g / LINES, r = g - dv * LINES;  // r = el * NF + j
     const int d = dv / NV, v = dv - d * NV;
     if (r >= last) continue;
-    const double* x = sX + v * VS;
-    int st = 1;
-    if (d == 0) {
-      x += r * N;  // line j of an element starts at its node j * N
-    } else {
-      const int el = r / NF;
-      x += r + el * (ND - NF);
-      st = N;
-      if constexpr (D == 3) {
-        if (d == 1) x += (r - el * NF) / N * (N * N - N);
-        else st = N * N;
-      }
-    }
+    int st;
+    const double* x = sX + v * VS + tile_line<D, N, N>(d, r, st);
     double val[N], lo, hi;
 #pragma unroll
     for (int a = 0; a < N; ++a) val[a] = x[a * st];
@@ -361,7 +524,7 @@ __device__ __forceinline__ void write_traces_fp64(const MeshArgs& m, const Fixed
 }
 
 // Traces of a tile of elements held in shared memory sX[el][v][node] (compute type C, element
-// stride SXS) -> tr, FP32 and FP32-pair operators: a thread owns one (direction, side,
+// stride SXS) -> tr, FP32-pair operator: a thread owns one (direction, side,
 // variable, face node) combination, so its line of nodes, stride and interpolation weights
 // are set up once, and interpolates it for a run of the tile's elements (the runs split the
 // elements when the block has threads to spare); this halves the instruction count of this
@@ -408,20 +571,31 @@ __global__ void __launch_bounds__(Tile<D, N>::THREADS) trace_kernel(const TraceA
   constexpr int ND = T::ND, NV = T::NV, EPB = T::EPB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sX = reinterpret_cast<C*>(smem_raw);
+  using Nodes = TileNodes<D, N, 128>;
+  const Nodes sN(smem_raw);  // FP32 operator
   const int el = threadIdx.x / ND, node = threadIdx.x - el * ND;
   const int e0 = blockIdx.x * EPB;
   const int e = e0 + el;
   const int ne = (int)A.m.ne;
   if (e < ne) {
+    C u[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
-      sX[std::is_same<R, double>::value ? v * T::THREADS + (int)threadIdx.x : (el * NV + v) * ND + node] =
-          Arith<C>::from_double(A.u[(v * ne + e) * ND + node]);
+    for (int v = 0; v < NV; ++v) u[v] = Arith<C>::from_double(A.u[(v * ne + e) * ND + node]);
+    if constexpr (std::is_same<R, float>::value) {
+      sN.store(Nodes::at(threadIdx.x), u);
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        sX[std::is_same<R, double>::value ? v * T::THREADS + (int)threadIdx.x
+                                          : (el * NV + v) * ND + node] = u[v];
+    }
   }
   __syncthreads();
   typename Arith<R>::S* tr = reinterpret_cast<typename Arith<R>::S*>(A.tr);
   if constexpr (std::is_same<R, double>::value)
     write_traces_fp64<D, N, 128>(A.m, A.ft, A.tab, sX, T::THREADS, e0, tr);
+  else if constexpr (std::is_same<R, float>::value)
+    write_traces_fp32<D, N, 128>(A.m, A.ft, sN, e0, tr);
   else
     write_traces<D, N, R, 128, C, NV * ND>(A.m, A.tab, sX, e0, tr);
 }
@@ -516,38 +690,43 @@ struct Update<double> {
   }
 };
 
-// Pointwise fluxes of a tile in shared memory: [EPB][D][NV][ND] values of R, except for
-// the 2D FP32 pairs, which keep pairs of variables together for the packed sweeps:
-// [EPB][D][NV/2][ND] of float4 {hi_v, hi_v+1, lo_v, lo_v+1}.  (In 3D the odd variable
-// count and the larger tiles cost more registers than the packing saves.)
+// Pointwise fluxes of a tile in shared memory.  FP32: D NodeArrays of the tile's nodes (then in
+// place the contributions of the direction's sweep and lift, then in the first one the next
+// stage input).  FP32 pairs: [EPB][D][NV][ND] of R, in 2D pairs of variables
+// together for the packed sweeps, [EPB][D][NV/2][ND] of float4 {hi_v, hi_v+1, lo_v, lo_v+1}
+// (in 3D the odd variable count and the larger tiles cost more registers than the packing
+// saves); the trace epilogue reuses them.
 template <int D, typename R> struct PackedSweeps { static constexpr bool value = false; };
 template <> struct PackedSweeps<2, df64> { static constexpr bool value = true; };
 template <int D, int N, typename R, int TT>
 constexpr size_t vol_flux_bytes() {
   using T = Tile<D, N, TT>;
   using C = typename TraceCompute<R>::C;
+  if (std::is_same<R, float>::value) return D * TileNodes<D, N, TT>::BYTES;
   const size_t f = PackedSweeps<D, R>::value ? sizeof(float4) * T::EPB * D * ((T::NV + 1) / 2) * T::ND
-                                             : sizeof(R) * T::EPB * sf_stride<D, N, R>();
-  const size_t x = sizeof(C) * T::EPB * sx_stride<D, N, C>();  // reused for the next input
+                                             : sizeof(R) * T::EPB * D * T::NV * T::ND;
+  const size_t x = sizeof(C) * T::EPB * T::NV * T::ND;  // reused for the next input
   return f > x ? f : x;
 }
 
 // Shared memory of the volume kernel: the pointwise fluxes of the tile, then (kStage) the
 // per-thread staging slots of the RK operands (FP64 solution; stage register in the
 // operator's storage type), then (kFaces) the numerical fluxes on every face of every
-// element of the tile, [EPB][D][side][NV][NF] values of R.  The trace epilogue reuses the
-// flux area.
+// element of the tile, [EPB][D][side][NV][NF] values of R (FP32: a NodeArray over
+// [EPB][D][side][NF]).
 template <int D, int N, typename R, int TT, bool kStage, bool kFaces = false>
 struct VolSmem {
   using T = Tile<D, N, TT>;
-  static constexpr size_t FLUX = vol_flux_bytes<D, N, R, TT>();
-  static constexpr size_t W_OFF = (FLUX + 15) / 16 * 16;
+  static constexpr size_t FLUX = (vol_flux_bytes<D, N, R, TT>() + 15) / 16 * 16;
+  static constexpr size_t W_OFF = FLUX;
   static constexpr size_t Q_OFF = W_OFF + sizeof(double) * T::NV * T::THREADS;
   static constexpr size_t STAGED =
       kStage ? Q_OFF + sizeof(typename Arith<R>::S) * T::NV * T::THREADS : FLUX;
   static constexpr size_t FACE_OFF = (STAGED + 15) / 16 * 16;
-  static constexpr size_t BYTES =
-      kFaces ? FACE_OFF + sizeof(R) * T::EPB * 2 * D * T::NV * T::NF : STAGED;
+  static constexpr size_t FACES = std::is_same<R, float>::value
+                                      ? NodeArray<D, T::EPB * 2 * D * T::NF>::BYTES
+                                      : sizeof(R) * T::EPB * 2 * D * T::NV * T::NF;
+  static constexpr size_t BYTES = kFaces ? FACE_OFF + FACES : STAGED;
 };
 
 // Where the volume kernel takes the numerical fluxes of its elements' faces from.
@@ -587,8 +766,8 @@ __device__ __forceinline__ void element_face_fluxes(const ElementFaces& F, const
                                                     bool active, unsigned char* face_smem);
 
 template <int D, int N, typename R, int TT, bool kStage = false, typename Faces = SplitFaces>
-__device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned char* smem_raw,
-                                         const Faces& faces = Faces()) {
+__device__ __forceinline__ void vol_body(const VolArgs& A, const SweepArg<D, N, R>& tab, int tile,
+                                         unsigned char* smem_raw, const Faces& faces = Faces()) {
   using T = Tile<D, N, TT>;
   using S = typename Arith<R>::S;
   constexpr bool kFaces = std::is_same<Faces, ElementFaces>::value;
@@ -605,17 +784,17 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned ch
     vbar = bars;
   }
   constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB;
-  using CT = typename TraceCompute<R>::C;
-  constexpr int SFS = sf_stride<D, N, R>(), SXS = sx_stride<D, N, CT>();
-  static_assert(sizeof(CT) * EPB * SXS <= SM::FLUX, "the next stage input fits the flux area");
-  R* sF = reinterpret_cast<R*>(smem_raw);  // [EPB][D][NV][ND], element stride SFS (packed sweeps: sF4 below)
+  constexpr bool kF32 = std::is_same<R, float>::value;
+  constexpr int SFS = D * NV * ND, SXS = NV * ND;  // element strides of sF and sX
+  using Nodes = TileNodes<D, N, TT>;
+  R* sF = reinterpret_cast<R*>(smem_raw);  // [EPB][D][NV][ND] (packed sweeps: sF4 below; FP32: Nodes)
   double* sW = reinterpret_cast<double*>(smem_raw + SM::W_OFF);  // [NV][THREADS] (kStage)
   S* sQ = reinterpret_cast<S*>(smem_raw + SM::Q_OFF);            // [NV][THREADS] (kStage)
   const int el = threadIdx.x / ND, node = threadIdx.x - el * ND;
   const int e0 = tile * EPB;
   const int ne = (int)A.m.ne;
   const int e = e0 + el;
-  const bool active = e < ne;
+  const bool active = el < EPB && e < ne;
 
   int ix[3] = {node % N, (node / N) % N, node / (N * N)};
   int ec[3] = {0, 0, 0};
@@ -707,7 +886,12 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned ch
   {
     R F[D][NV];
     euler_flux_all<D, R>(u, Arith<R>::pair(A.gm1, A.gm1f), F);
-    if constexpr (PackedSweeps<D, R>::value) {
+    if constexpr (kF32) {
+      if (active) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) Nodes(smem_raw + d * Nodes::BYTES).store(Nodes::at(tid), F[d]);
+      }
+    } else if constexpr (PackedSweeps<D, R>::value) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
 #pragma unroll
@@ -731,7 +915,80 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned ch
 #pragma unroll
   for (int v = 0; v < NV; ++v) acc[v] = acc_zero(Acc());
   const S* fl = reinterpret_cast<const S*>(A.fl);
-  if (active) {
+  if constexpr (kF32) {
+    // One direction after the other, in place in the first one's NodeArray: one thread per
+    // (line, variable pair), the pairs of a line in neighbouring lanes, with the table in the
+    // constant bank (one thread per node would read every value N times and its table rows:
+    // the shared-memory data pipe, which bounds this kernel, moves about half as much).  The
+    // lift follows per node.  Every sum keeps the order of one thread per node (directions,
+    // then lifts), and with it its bits.  Us per stage, element path, against that form with
+    // one 4-byte access per value and variable: 256^2 p=4 54.6 -> 47.7, 432^2 p=2 67 -> 56,
+    // 320^2 p=3 58 -> 43, 160^2 p=7 68 -> 41; 64^3 p=2 474 -> 424, 48^3 p=3 350 -> 289, 32^3
+    // p=5 423 -> 329.
+    constexpr int LINES = EPB * NF, BLOCK = vol_block<R>(T::THREADS), USED = (2 * LINES + 31) / 32 * 32;
+    const int last = (ne - e0) * NF;
+    const Nodes Y(smem_raw);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const Nodes X(smem_raw + d * Nodes::BYTES);
+      for (int g = tid; g < 2 * LINES; g += BLOCK) {
+        const int r = g >> 1, pr = g & 1;
+        if (r >= last) continue;
+        int st;
+        const int base = tile_line<D, N, Nodes::PN>(d, r, st);
+        float2 x[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) x[a] = X.pair(base + a * st, pr);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          float2 s = d > 0 ? Y.pair(base + i * st, pr) : make_float2(0.0f, 0.0f);
+#pragma unroll
+          for (int a = 0; a < N; ++a) s = __ffma2_rn(tab.q[d][i * N + a], x[a], s);
+          Y.pair(base + i * st, pr) = s;
+        }
+      }
+      if constexpr (D == 3) {  // the fifth variable, from the warp after the pairs' last one on
+        int g = tid - USED % BLOCK;
+        if (g < 0) g += BLOCK;
+        for (; g < LINES; g += BLOCK) {
+          if (g >= last) continue;
+          int st;
+          const int base = tile_line<D, N, Nodes::PN>(d, g, st);
+          float x[N];
+#pragma unroll
+          for (int a = 0; a < N; ++a) x[a] = X.b()[base + a * st];
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            float s = d > 0 ? Y.b()[base + i * st] : 0.0f;
+#pragma unroll
+            for (int a = 0; a < N; ++a) s = fmaf(tab.q[d][i * N + a].x, x[a], s);
+            Y.b()[base + i * st] = s;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (active) {
+      Y.load(Nodes::at(tid), acc);
+      const NodeArray<D, EPB * 2 * D * NF> G(smem_raw + SM::FACE_OFF);  // face fluxes (kFaces)
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const int j = face_index<D, N>(d, ix);
+        const float lm = (A.scaled ? A.tab->Lmsf[d] : A.tab->Lmf[d])[ix[d]].x;
+        const float lp = (A.scaled ? A.tab->Lpsf[d] : A.tab->Lpf[d])[ix[d]].x;
+        float flo[NV], fhi[NV];
+        if constexpr (kFaces) {
+          G.load((el * 2 * D + 2 * d) * NF + j, flo);
+          G.load((el * 2 * D + 2 * d + 1) * NF + j, fhi);
+        } else {
+          load_flux<D, N>(fl, ne, d, elem_shift(A.m, e, ec, d, -1), j, flo);
+          load_flux<D, N>(fl, ne, d, e, j, fhi);
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = fmaf(-lp, fhi[v], fmaf(lm, flo[v], acc[v]));
+      }
+    }
+  } else if (active) {
     df64acc2 acc2[NP];  // packed sweeps: lane k of pair pr accumulates variable 2 pr + k
 #pragma unroll
     for (int pr = 0; pr < NP; ++pr) acc2[pr] = acc2_zero();
@@ -823,7 +1080,14 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, int tile, unsigned ch
   }
 
   // 4. traces of the next stage input
-  if (A.write_traces) {
+  if constexpr (kF32) {
+    if (A.write_traces) {
+      const Nodes sX(smem_raw);  // over this thread's own values
+      if (active) sX.store(Nodes::at(tid), xnext);
+      __syncthreads();
+      write_traces_fp32<D, N, TT>(A.m, A.ft, sX, e0, reinterpret_cast<float*>(A.tr));
+    }
+  } else if (A.write_traces) {
     __syncthreads();
     C* sX = reinterpret_cast<C*>(smem_raw);  // reuse: [EPB][NV][ND], element stride SXS
 #pragma unroll
@@ -1119,17 +1383,19 @@ template <int D, int N> struct VolKernelRegs<D, N, double> {
   static constexpr int value = D == 2 ? 48 : 64;
 };
 template <int D, int N> struct VolKernelRegs<D, N, float> {
-  static constexpr int value = (D == 2 && N != 3 && N != 4 && N != 6) ? 32 : 40;  // no spills (ptxas, sm_103a)
+  // 2D: 40 registers are 1 to 4 % slower (N = 8: 1 % faster); 3D: 32 spill (2 to 4 % slower),
+  // 48 cost up to 8 %
+  static constexpr int value = D == 2 && N != 8 ? 32 : 40;
 };
 
 template <int D, int N, typename R, int TT = 128>
-__global__ void __launch_bounds__(Tile<D, N, TT>::THREADS,
+__global__ void __launch_bounds__(vol_block<R>(Tile<D, N, TT>::THREADS),
                                   min_blocks_for(VolKernelRegs<D, N, R>::value,
-                                                 Tile<D, N, TT>::THREADS))
-vol_kernel(const VolArgs A) {
+                                                 vol_block<R>(Tile<D, N, TT>::THREADS)))
+vol_kernel(const __grid_constant__ VolArgs A, const __grid_constant__ SweepArg<D, N, R> tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dependency();
-  vol_body<D, N, R, TT, VolStages<R>::value>(A, blockIdx.x, smem_raw);
+  vol_body<D, N, R, TT, VolStages<R>::value>(A, tab, blockIdx.x, smem_raw);
 }
 
 // (64, 192 and 256 threads: 2 to 25 % slower than 128 over the degrees)
@@ -1243,16 +1509,18 @@ __device__ __forceinline__ void flux_body(const FluxArgs& A, int bx, int d) {
   const int ehi = elem_shift(A.m, e, ec, d, +1);
   const S* tr = reinterpret_cast<const S*>(A.tr);
   R wm[NV], wp[NV], f[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    wm[v] = Arith<R>::load(tr + (((d * 2 + 1) * NV + v) * ne + e) * NF + j);
-    wp[v] = Arith<R>::load(tr + (((d * 2 + 0) * NV + v) * ne + ehi) * NF + j);
-  }
+  load_traces<D, N, R>(tr, ne, d * 2 + 1, e, j, wm);
+  load_traces<D, N, R>(tr, ne, d * 2, ehi, j, wp);
   const int slot = A.pe_mode ? A.pe_slot[d * ne + e] : -1;
   face_flux<D, N, R>(A, d, slot, j, wm, wp, true, f);
   S* fl = reinterpret_cast<S*>(A.fl);
+  using Lay = FluxLay<D, N, R>;
+  if constexpr (TraceLay<D, N, R>::kTogether && D == 2) {
+    *reinterpret_cast<float4*>(fl + Lay::at(ne, d, 0, e, j)) = make_float4(f[0], f[1], f[2], f[3]);
+  } else {
 #pragma unroll
-  for (int v = 0; v < NV; ++v) Arith<R>::store(fl + ((d * NV + v) * ne + e) * NF + j, f[v]);
+    for (int v = 0; v < NV; ++v) Arith<R>::store(fl + Lay::at(ne, d, v, e, j), f[v]);
+  }
 }
 
 // Numerical fluxes on the 2D faces of element e (tile slot el) into shared memory
@@ -1277,34 +1545,35 @@ __device__ __forceinline__ void element_face_fluxes(const ElementFaces& F, const
     const int nb = elem_shift(m, e, ec, d, side ? 1 : -1);
     const int lo = side ? e : nb, hi = side ? nb : e;
     R wm[NV], wp[NV], f[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      wm[v] = Arith<R>::load(tr + (((d * 2 + 1) * NV + v) * ne + lo) * NF + j);
-      wp[v] = Arith<R>::load(tr + (((d * 2 + 0) * NV + v) * ne + hi) * NF + j);
-    }
+    load_traces<D, N, R>(tr, ne, d * 2 + 1, lo, j, wm);
+    load_traces<D, N, R>(tr, ne, d * 2, hi, j, wp);
     const int slot = F.f.pe_mode ? F.f.pe_slot[d * ne + lo] : -1;
     face_flux<D, N, R>(F.f, d, slot, j, wm, wp, side == 1, f);
+    if constexpr (std::is_same<R, float>::value) {
+      NodeArray<D, T::EPB * 2 * D * NF>(face_smem).store((el * 2 * D + ds) * NF + j, f);
+    } else {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sFace[(ds * NV + v) * NF + j] = f[v];
+      for (int v = 0; v < NV; ++v) sFace[(ds * NV + v) * NF + j] = f[v];
+    }
   }
 }
 
 // One launch per RK stage without the face-flux launch: the volume kernel with every
 // element evaluating the numerical fluxes on its own faces (ElementFaces).  Register
-// budgets: no spills (ptxas sm_103a); the FP32 form measured best at 48 (40 spilled and
-// lost 8 %, 56 gained nothing).
+// budgets: no spills (ptxas sm_103a); the FP32 form measured best at 48 over the degrees (40:
+// up to 30 % slower, 56: 1 to 5 %).
 template <int D, int N, typename R> struct VolFacesRegs { static constexpr int value = D == 2 ? 64 : 80; };
 template <int D, int N> struct VolFacesRegs<D, N, float> { static constexpr int value = 48; };
 template <int D, int N> struct VolFacesRegs<D, N, double> { static constexpr int value = D == 2 ? 72 : 80; };
 
 template <int D, int N, typename R, int TT = 128>
-__global__ void __launch_bounds__(Tile<D, N, TT>::THREADS,
+__global__ void __launch_bounds__(vol_block<R>(Tile<D, N, TT>::THREADS),
                                   min_blocks_for(VolFacesRegs<D, N, R>::value,
-                                                 Tile<D, N, TT>::THREADS))
-vol_faces_kernel(const FusedArgs A) {
+                                                 vol_block<R>(Tile<D, N, TT>::THREADS)))
+vol_faces_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ SweepArg<D, N, R> tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   grid_dependency();
-  vol_body<D, N, R, TT, VolStages<R>::value, ElementFaces>(A.v, blockIdx.x, smem_raw,
+  vol_body<D, N, R, TT, VolStages<R>::value, ElementFaces>(A.v, tab, blockIdx.x, smem_raw,
                                                            ElementFaces{A.f, A.tr_in, A.err});
 }
 
@@ -1344,15 +1613,16 @@ template <int D, int N, typename R>
 cudaError_t launch_trace_t(const TraceArgs& a, cudaStream_t s) {
   using T = Tile<D, N>;
   const int64_t blocks = (a.m.ne + T::EPB - 1) / T::EPB;
-  const size_t smem = sizeof(R) * T::EPB * T::NV * T::ND;
+  const size_t smem = std::is_same<R, float>::value ? TileNodes<D, N, 128>::BYTES
+                                                    : sizeof(R) * T::EPB * T::NV * T::ND;
   trace_kernel<D, N, R><<<(unsigned)blocks, T::THREADS, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 // Launch that may start while the previous kernel of the stream runs (grid_dependency).
-template <typename A>
-cudaError_t launch_dependent(void (*kernel)(A), unsigned gx, unsigned gy, int threads, size_t smem,
-                             cudaStream_t s, const A& args) {
+template <typename... A>
+cudaError_t launch_dependent(void (*kernel)(A...), unsigned gx, unsigned gy, int threads, size_t smem,
+                             cudaStream_t s, const A&... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -1363,7 +1633,7 @@ cudaError_t launch_dependent(void (*kernel)(A), unsigned gx, unsigned gy, int th
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Opt-in for more than 48 KB of dynamic shared memory.
@@ -1388,7 +1658,8 @@ cudaError_t launch_vol_t(const VolArgs& a, cudaStream_t s) {
   } else {
     const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value>::BYTES;
     if ((err = allow_smem(vol_kernel<D, N, R>, smem)) != cudaSuccess) return err;
-    return launch_dependent(vol_kernel<D, N, R>, blocks, 1, T::THREADS, smem, s, a);
+    return launch_dependent(vol_kernel<D, N, R>, blocks, 1, vol_block<R>(T::THREADS), smem, s, a,
+                            sweep_arg<D, N, R>(a));
   }
 }
 
@@ -1406,7 +1677,8 @@ cudaError_t launch_vol_faces_t(const FusedArgs& a, cudaStream_t s) {
   } else {
     const size_t smem = VolSmem<D, N, R, TT, VolStages<R>::value, true>::BYTES;
     if ((err = allow_smem(vol_faces_kernel<D, N, R, TT>, smem)) != cudaSuccess) return err;
-    return launch_dependent(vol_faces_kernel<D, N, R, TT>, blocks, 1, T::THREADS, smem, s, a);
+    return launch_dependent(vol_faces_kernel<D, N, R, TT>, blocks, 1, vol_block<R>(T::THREADS), smem, s,
+                            a, sweep_arg<D, N, R>(a.v));
   }
 }
 

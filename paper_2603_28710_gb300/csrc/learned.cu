@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(128) learned_apply_kernel(const LearnArgs A) {
   S* fl = reinterpret_cast<S*>(A.fl);
   const int ne = (int)A.m.ne;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) Arith<R>::store(fl + ((d * NV + v) * ne + e) * NF + j, f[v]);
+  for (int v = 0; v < NV; ++v) Arith<R>::store(fl + FluxLay<D, N, R>::at(ne, d, v, e, j), f[v]);
 }
 
 // thread per (side, var, slot, face node): PE-face traces of the current stage input
@@ -159,8 +159,8 @@ __global__ void log_kernel(const typename Arith<R>::S* tr, const int32_t* face_d
   const int eh = elem_shift(m, e, ec, d, +1);
   const int ne = (int)m.ne;
   // side 0: high-side trace of e (minus state), side 1: low-side trace of its neighbour
-  const int idx = side == 0 ? (((d * 2 + 1) * NV + v) * ne + e) * NF + j
-                            : (((d * 2 + 0) * NV + v) * ne + eh) * NF + j;
+  using Lay = TraceLay<D, N, R>;
+  const int idx = side == 0 ? Lay::at(ne, d * 2 + 1, v, e, j) : Lay::at(ne, d * 2, v, eh, j);
   out[g] = Arith<R>::to_double(Arith<R>::load(tr + idx));
 }
 

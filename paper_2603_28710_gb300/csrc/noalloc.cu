@@ -37,7 +37,7 @@ adg_status noalloc_fail(adg_status st, const std::string& m) {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // The operator tables travel as a kernel argument (kernel arguments may hold up to 32 KB;
-// the tables take about 13 KB) and a one-block kernel stores them into the scratch array:
+// the tables take about 17 KB) and a one-block kernel stores them into the scratch array:
 // the launch copies the argument when it is enqueued, so no host memory is read after the
 // call returns and no host-to-device copy waits for the stream.
 struct TableBlob {
