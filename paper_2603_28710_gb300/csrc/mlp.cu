@@ -86,18 +86,28 @@ __device__ __forceinline__ void ldmatrix_trans(unsigned (&r)[4], const uint16_t*
                : "memory");
 }
 
+// the same without the transposition
+__device__ __forceinline__ void ldmatrix(unsigned (&r)[4], const uint16_t* row) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(row))
+               : "memory");
+}
+
 // First-layer activations tanh(W1 x + b1) of the 16-column block kk for rows g and g+8: h[row]
-// [columns c, c+1, c+8, c+9], c = 16 kk + 2t.  w: W1[64][4] | b1[64].
+// [columns c, c+1, c+8, c+9], c = 16 kk + 2t.  w: W1[64][4] | b1[64], 16-byte aligned.
 __device__ __forceinline__ void first_layer(const float* w, const float (&x0)[4], const float (&x1)[4],
                                             int kk, int t, float (&h)[2][4]) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int c = kk * 16 + 2 * t + (q & 1) + (q >> 1) * 8;
+    const float4 w1 = *reinterpret_cast<const float4*>(w + kW1 + c * 4);
+    const float wc[4] = {w1.x, w1.y, w1.z, w1.w};
     float z0 = w[kB1 + c], z1 = w[kB1 + c];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      z0 = fmaf(w[kW1 + c * 4 + i], x0[i], z0);
-      z1 = fmaf(w[kW1 + c * 4 + i], x1[i], z1);
+      z0 = fmaf(wc[i], x0[i], z0);
+      z1 = fmaf(wc[i], x1[i], z1);
     }
     h[0][q] = tanhf(z0);
     h[1][q] = tanhf(z1);
@@ -398,19 +408,26 @@ mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
 
 // ---- inference -------------------------------------------------------------------------
 constexpr int kInferWarps = 4;
+constexpr int kInferBlocks = 7;  // per SM (72 registers; at 8 it spills, 9 are 13 % slower)
 
-__global__ void __launch_bounds__(32 * kInferWarps)
+// A warp per 16 samples.  Bound by the issue of the tanh code; the hidden layer's weights were
+// it before: rows of 128 bytes put the eight rows of a B fragment on the same banks (8-fold
+// conflicts, 72 % of the time in shared-memory wavefronts).  Padded rows and ldmatrix, two
+// column blocks each: 1.97 M samples 456 -> 239 us, 65536 25 -> 15.5 us, the same bits.
+__global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks)
 mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x, int n,
                        float* __restrict__ y) {
-  __shared__ float Wf[kW2];                  // W1 | b1 (FP32)
-  __shared__ float Wo[kMlpParams - kB2];     // b2 | w3 | b3 (FP32)
-  __shared__ __align__(16) uint16_t W2[64 * 64];  // [n = out][k = in], BF16
+  __shared__ __align__(16) float Wf[kW2];               // W1 | b1 (FP32)
+  __shared__ __align__(16) float Wo[kMlpParams - kB2];  // b2 | w3 | b3 (FP32)
+  __shared__ __align__(16) uint16_t W2[64][kPitch];     // [out][in], BF16
   for (int i = threadIdx.x; i < kW2; i += blockDim.x) Wf[i] = bf16_to_float(pbf[i]);
   for (int i = threadIdx.x; i < kMlpParams - kB2; i += blockDim.x) Wo[i] = bf16_to_float(pbf[kB2 + i]);
-  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) W2[i] = pbf[kW2 + i];
+  for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) W2[i >> 6][i & 63] = pbf[kW2 + i];
   __syncthreads();
-  const unsigned* W2w = reinterpret_cast<const unsigned*>(W2);  // pairs along k
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // B fragments of two 8-column blocks per ldmatrix: tile m = lane / 8 holds the rows (outputs)
+  // of block m / 2 and the inputs 8 (m % 2) to 8 (m % 2) + 7 of the k-step
+  const uint16_t* w2row = &W2[(lane >> 4) * 8 + (lane & 7)][((lane >> 3) & 1) * 8];
   const int tiles = (n + 15) / 16;
   for (int tile = blockIdx.x * kInferWarps + (threadIdx.x >> 5); tile < tiles;
        tile += gridDim.x * kInferWarps) {
@@ -433,27 +450,30 @@ mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict
       unsigned a[3][4];
       split_fragment(h, a);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int nrow = j * 8 + g;  // output unit of this lane's B column
-        const unsigned b0 = W2w[(nrow * 64 + kk * 16 + 2 * t) >> 1];
-        const unsigned b1 = W2w[(nrow * 64 + kk * 16 + 2 * t + 8) >> 1];
-        mma_bf16(acc[j], a[0], b0, b1);
-        mma_bf16(acc[j], a[1], b0, b1);
-        mma_bf16(acc[j], a[2], b0, b1);
+      for (int j = 0; j < 8; j += 2) {
+        unsigned b[4];
+        ldmatrix(b, w2row + j * 8 * kPitch + kk * 16);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          mma_bf16(acc[j + i], a[0], b[2 * i], b[2 * i + 1]);
+          mma_bf16(acc[j + i], a[1], b[2 * i], b[2 * i + 1]);
+          mma_bf16(acc[j + i], a[2], b[2 * i], b[2 * i + 1]);
+        }
       }
     }
     // second activation and the output layer: this lane holds columns 2t, 2t+1 of each
     // 8-column block for rows r0 (acc[j][0..1]) and r1 (acc[j][2..3])
     float y0 = 0.0f, y1 = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int c = j * 8 + 2 * t + q;
-        const float w3 = Wo[kW3 - kB2 + c], b2 = Wo[c];
-        y0 = fmaf(w3, tanhf(acc[j][q] + b2), y0);
-        y1 = fmaf(w3, tanhf(acc[j][2 + q] + b2), y1);
-      }
+    for (int j = 0; j < 8; ++j) {
+      const int c = j * 8 + 2 * t;
+      const float2 b2 = *reinterpret_cast<const float2*>(&Wo[c]);
+      const float2 w3 = *reinterpret_cast<const float2*>(&Wo[kW3 - kB2 + c]);
+      y0 = fmaf(w3.x, tanhf(acc[j][0] + b2.x), y0);
+      y1 = fmaf(w3.x, tanhf(acc[j][2] + b2.x), y1);
+      y0 = fmaf(w3.y, tanhf(acc[j][1] + b2.y), y0);
+      y1 = fmaf(w3.y, tanhf(acc[j][3] + b2.y), y1);
+    }
     y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
     y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
     y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
@@ -496,7 +516,7 @@ cudaError_t mlp_infer(const uint16_t* params, const float* x, int64_t n, float* 
   if (n <= 0) return cudaSuccess;
   const int64_t tiles = (n + 15) / 16;
   const int64_t want = (tiles + kInferWarps - 1) / kInferWarps;
-  const int blocks = (int)(want < 152 * 16 ? want : 152 * 16);
+  const int blocks = (int)(want < 152 * kInferBlocks ? want : 152 * kInferBlocks);
   mlp_forward_mma_kernel<<<blocks, 32 * kInferWarps, 0, s>>>(params, x, (int)n, y);
   return cudaGetLastError();
 }
