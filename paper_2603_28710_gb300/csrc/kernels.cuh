@@ -794,7 +794,9 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, const SweepArg<D, N, 
   const int e0 = tile * EPB;
   const int ne = (int)A.m.ne;
   const int e = e0 + el;
-  const bool active = el < EPB && e < ne;
+  // (the test of el where the block has no spare threads costs the 3D pairs 6 %: 48^3 p=3 788 ->
+  // 835 us)
+  const bool active = (vol_block<R>(T::THREADS) == T::THREADS || el < EPB) && e < ne;
 
   int ix[3] = {node % N, (node / N) % N, node / (N * N)};
   int ec[3] = {0, 0, 0};
