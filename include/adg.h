@@ -223,7 +223,8 @@ adg_status adg_get_profile(adg_solver* s, double* ms, int64_t* launches);
 
 /* ---- operator without device allocation ------------------------------------------ */
 
-/* Size of the built-in device scratch array used by adg_rhs_noalloc (32 MiB). */
+/* Scratch limit of adg_rhs_noalloc (32 MiB; the built-in device array that holds the scratch is
+ * a few KB larger). */
 #define ADG_NOALLOC_SCRATCH_BYTES (32u << 20)
 
 /* The synchronous FP64 operator k = M^{-1} L_h(u) of adg_rhs, for callers that cannot
@@ -234,8 +235,7 @@ adg_status adg_get_profile(adg_solver* s, double* ms, int64_t* launches);
  *
  * Needs no handle and allocates nothing: no cudaMalloc, no cudaFree, no allocating
  * library routine.  Its scratch (operator tables, face traces, face fluxes) sits in one
- * file-scope device array of ADG_NOALLOC_SCRATCH_BYTES that every GPU loading the library
- * holds until the process exits.  The first call on a device looks up that array's
+ * file-scope device array that every GPU loading the library holds until the process exits.  The first call on a device looks up that array's
  * device address (cudaGetSymbolAddress, with the device current); make that first call
  * before any stream capture.  Every call overwrites all the scratch it later reads, so
  * nothing carries over between calls; calls that overlap on the GPU (two streams, two
@@ -250,7 +250,7 @@ adg_status adg_get_profile(adg_solver* s, double* ms, int64_t* launches);
  * a kernel argument and a kernel stores them into the scratch array, so no host memory is
  * read after the call returns and no copy from pageable memory stalls the host.  A mesh
  * whose scratch
- * (2 d + d) (d+2) n_elements (degree+1)^(d-1) doubles plus the tables exceeds
+ * (2 d + d) (d+2) n_elements (degree+1)^(d-1) doubles plus 8960 bytes (tables) exceeds
  * ADG_NOALLOC_SCRATCH_BYTES is rejected with ADG_ERR_INVALID; adg_last_error(NULL) says
  * how many bytes it needed.  Other errors: ADG_ERR_INVALID (arguments), ADG_ERR_CUDA. */
 adg_status adg_rhs_noalloc(const adg_mesh* mesh, int degree, double gamma, const double* u,

@@ -22,8 +22,13 @@ void noalloc_set_error(const char* msg);
 
 namespace {
 
+// The limit counts 8960 bytes for the tables; what the fixed-point tables take beyond them lies
+// past it, so that the meshes that fit do not depend on the tables' size.
 constexpr size_t kScratchBytes = (size_t)ADG_NOALLOC_SCRATCH_BYTES;
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+constexpr size_t kCountedTables = 8960;
+constexpr size_t kTableBytes = (sizeof(adg::OpTables) + 255) & ~(size_t)255;
+static_assert(kTableBytes >= kCountedTables, "the scratch array holds the limit and the tables' excess");
+static __device__ __align__(256) unsigned char g_scratch[kScratchBytes + kTableBytes - kCountedTables];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -74,10 +79,9 @@ extern "C" adg_status adg_rhs_noalloc(const adg_mesh* mesh, int degree, double g
   }
   if (count != (int64_t)NV * ne * ND) return noalloc_fail(ADG_ERR_INVALID, "count does not match the mesh");
   // scratch layout: tables | traces [d][side][v][e][j] | fluxes [d][v][e][j]
-  const size_t tab_bytes = align256(sizeof(OpTables));
   const size_t tr_bytes = align256((size_t)2 * dim * NV * ne * NF * sizeof(double));
   const size_t fl_bytes = align256((size_t)dim * NV * ne * NF * sizeof(double));
-  const size_t need = tab_bytes + tr_bytes + fl_bytes;
+  const size_t need = kCountedTables + tr_bytes + fl_bytes;
   if (need > kScratchBytes)
     return noalloc_fail(ADG_ERR_INVALID,
                         "mesh too large for the built-in scratch: needs " + std::to_string(need) +
@@ -106,8 +110,8 @@ extern "C" adg_status adg_rhs_noalloc(const adg_mesh* mesh, int degree, double g
   std::memset(&tab, 0, sizeof(tab));
   noalloc_build_tables(dim, N, h, &tab);
   OpTables* tab_dev = reinterpret_cast<OpTables*>(base);
-  void* tr = base + tab_bytes;
-  void* fl = base + tab_bytes + tr_bytes;
+  void* tr = base + kTableBytes;
+  void* fl = base + kTableBytes + tr_bytes;
   TableBlob blob;
   std::memcpy(blob.v, &tab, sizeof(OpTables));
   store_tables_kernel<<<1, 128, 0, s>>>(blob, reinterpret_cast<unsigned long long*>(tab_dev));
