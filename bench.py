@@ -72,6 +72,13 @@ def vol_flops_per_node(D=2, N=DEGREE + 1):
     return pointwise + sweeps + lift + rk + traces
 
 
+def vol_fp64_ops_per_node(D):
+    """FP64 operations the FP64 volume kernel runs per node on the FP64 pipe: pointwise flux
+    (reciprocal 3, velocities, kinetic energy, pressure and enthalpy, flux columns) and the RK
+    update; its contractions run in fixed point on the integer pipe."""
+    return 6 + 3 * D + D * (D + 1) // 2 + 2 * (D + 2)
+
+
 Q_BYTES = {"fp64": 8, "df64": 8, "fp32": 4}  # storage of the 2N register q per value
 
 
@@ -92,8 +99,8 @@ def kernel_source_hash(precision):
     from (a profile taken on other sources no longer describes them)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2603_28710_gb300", "csrc")
-    for name in ("adg_internal.h", "arith.cuh", "df64.cuh", "kernels.cuh", f"k_{precision}.cu",
-                 f"kv_{precision}.cu"):
+    for name in ("adg_internal.h", "arith.cuh", "df64.cuh", "fixline.cuh", "kernels.cuh",
+                 f"k_{precision}.cu", f"kv_{precision}.cu"):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(name.encode())
             h.update(f.read())
@@ -301,17 +308,29 @@ def whole_job_value(work_per_rank_per_step, steps, seconds_max, world):
     return world * work_per_rank_per_step * steps / seconds_max / 1e9
 
 
-def vol_kernel_name(precision, D, N):
-    """The volume/update kernel the default path (ADG_PATH_AUTO) runs for an arithmetic:
-    the element-face kernel for FP32, the split path's volume kernel otherwise."""
-    return f"{'vol_faces_kernel' if precision == 'fp32' else 'vol_kernel'}<{D},{N}>"
+def default_path(precision, N, nodes):
+    """The kernel path ADG_PATH_AUTO takes on large meshes: split, except for FP32 with four
+    nodes per direction or fewer than 2^20 nodes (element)."""
+    return "element" if precision == "fp32" and (N == 4 or nodes < 2 ** 20) else "split"
+
+
+def other_path(precision, N, nodes):
+    return "split" if default_path(precision, N, nodes) == "element" else "element"
+
+
+def vol_kernel_name(precision, D, N, nodes):
+    """The volume/update kernel the default path runs for an arithmetic."""
+    name = "vol_faces_kernel" if default_path(precision, N, nodes) == "element" else "vol_kernel"
+    return f"{name}{'_fp64' if precision == 'fp64' else ''}<{D},{N}>"
 
 
 def roofline_line(precision, D, N, ndof, vol_ms, vol_n, mpk, kernel):
-    """Roofline of the volume/update kernel from its average launch time: algorithmic
-    flops (FP64 form, bound by the FP64 pipe) or algorithmic HBM bytes (FP32 and FP32-pair
-    forms) per launch over the average launch duration, against the rates measured on this
-    GPU (adg_measure_peak) and MEASURED_PEAKS.json's copy bandwidth."""
+    """Roofline of the volume/update kernel from its average launch time: the operations it
+    runs on the FP64 pipe (FP64 form, each counted as one FMA, 2 flops) or algorithmic HBM
+    bytes (FP32 and FP32-pair forms) per launch over the average launch duration, against the
+    rates measured on this GPU (adg_measure_peak) and MEASURED_PEAKS.json's copy bandwidth.
+    alu_view compares all algorithmic flops with the FP64 rate: above 1 where contractions run
+    in fixed point."""
     nodes = ndof // (D + 2)
     avg_s = vol_ms * 1e-3 / max(vol_n, 1)
     flops = vol_flops_per_node(D, N) * nodes
@@ -324,8 +343,8 @@ def roofline_line(precision, D, N, ndof, vol_ms, vol_n, mpk, kernel):
     alu_view = {"achieved_tflops": flops / avg_s / 1e12, "fp64_fma_peak_tflops": fp64,
                 "frac_of_fp64": (flops / avg_s / 1e12 / fp64) if fp64 else None}
     if precision == "fp64":
-        roof = {"bound": "alu", "achieved": flops / avg_s / 1e12, "peak": fp64 or 1.25,
-                "unit": "TFLOP/s",
+        roof = {"bound": "alu", "achieved": 2 * vol_fp64_ops_per_node(D) * nodes / avg_s / 1e12,
+                "peak": fp64 or 1.25, "unit": "TFLOP/s",
                 "peak_source": ("FP64 FMA rate measured in this run by adg_measure_peak (nominal 1.25)"
                                 if fp64 else "nominal FP64 1.25 TFLOP/s")}
     else:
@@ -557,7 +576,7 @@ def tgv_run(adg, stream, mpk, flush, k=3, total_steps=100, with_cpu=True):
                      "flux_ms_per_launch": prof["flux"][0] / max(prof["flux"][1], 1),
                      "kernel_path": "element" if prof["flux"][1] == 0 else "split",
                      "roofline": dict(roofline_line(prec, 3, TGV_DEGREE + 1, ndof, vol_ms, vol_n,
-                                                    mpk, vol_kernel_name(prec, 3, TGV_DEGREE + 1)),
+                                                    mpk, vol_kernel_name(prec, 3, TGV_DEGREE + 1, ndof // 5)),
                                       traffic=ncu_traffic(prec, "kernels_3d_traffic"),
                                       traffic_note="ncu capture at 48^3 scaled to 64^3 by the "
                                                    "element count"),
@@ -588,13 +607,13 @@ def tgv_run(adg, stream, mpk, flush, k=3, total_steps=100, with_cpu=True):
             out[prec][f"rel_l2_diff_vs_fp64_after_{total_steps}_steps"] = float(
                 np.linalg.norm(u - u64) / np.linalg.norm(u64))
         del u
-    # the fused per-stage kernel, and each arithmetic on the path its default does not take
-    # (element path for FP64 and pairs, split path for FP32), on the same workload (one
-    # schedule cycle per form)
+    # the fused per-stage kernel, and each arithmetic on the path its default does not take, on
+    # the same workload (one schedule cycle per form)
     out["fused_path"], out["other_path"] = {}, {}
     for key, prec, path in (("fused_path", "fp64", "fused"), ("fused_path", "df64", "fused"),
-                            ("fused_path", "fp32", "fused"), ("other_path", "fp64", "element"),
-                            ("other_path", "df64", "element"), ("other_path", "fp32", "split")):
+                            ("fused_path", "fp32", "fused"),
+                            *(("other_path", p, other_path(p, TGV_DEGREE + 1, ndof // 5))
+                              for p in ("fp64", "df64", "fp32"))):
         s = adg.Solver(dim=3, n_elem=(TGV_N,) * 3, degree=TGV_DEGREE, lo=(0, 0, 0),
                        hi=(2 * np.pi,) * 3, P=(TGV_P,) * 3, max_delay=TGV_L, flux="at", rk="ck45",
                        cfl=0.1, precision=prec, kernel_path=path, stream=stream.cuda_stream)
@@ -773,7 +792,7 @@ def run_gpu(args, rank, world, local_rank):
     vol_ms, vol_n = prof["vol"]
     flux_ms, flux_n = prof["flux"]
     roof = roofline_line(args.precision, 2, DEGREE + 1, ndof, vol_ms, vol_n, mpk,
-                         vol_kernel_name(args.precision, 2, DEGREE + 1))
+                         vol_kernel_name(args.precision, 2, DEGREE + 1, ndof // 4))
     roof["traffic"] = ncu_traffic(args.precision)
     launches_per_step = (vol_n + flux_n) / max(args.profile_steps, 1)
 
@@ -808,13 +827,12 @@ def run_gpu(args, rank, world, local_rank):
                                                 kernel_path="fused").items()
                    if k in ("value", "vol_ms_per_launch", "l2_error_vs_exact")}
             for prec in ("fp64", "df64", "fp32")}
-        # each arithmetic on the path the default does not take for it (the element path
-        # for FP64 and pairs, the split path for FP32)
+        # each arithmetic on the path the default does not take for it
         variants["other_path"] = {
             prec: {k: v for k, v in variant_run(adg, stream, prec, steps_per, 3, 1, dt,
                                                 kernel_path=path).items()
                    if k in ("value", "vol_ms_per_launch", "flux_ms_per_launch", "kernel_path")}
-            for prec, path in (("fp64", "element"), ("df64", "element"), ("fp32", "split"))}
+            for prec, path in ((p, other_path(p, DEGREE + 1, ndof // 4)) for p in ("fp64", "df64", "fp32"))}
 
     batched = None
     if world == 1 and not args.no_batch:

@@ -7,13 +7,13 @@
 //   flux_kernel : one thread per (direction, face, face node): numerical flux of Eq. 8-9
 //                 from the two stored traces; on faces between subdomains it applies the
 //                 delayed / AT rules of Algorithms 2-3 (Eq. 13-14) against a ring buffer.
-//   vol_kernel (FP64: vol_kernel_fp64) : one thread per node, a tile of elements per block: pointwise Euler flux
-//                 (Eq. 2), sum-factorised weak derivative along each direction, face lift,
-//                 inverse mass (diagonal for collocated Gauss points; folded into the
-//                 tables), the low-storage RK update (Eq. 10 or the 2N form), and the
-//                 face traces of the next stage input.
+//   vol_kernel (FP64: vol_kernel_fp64) : a tile of elements per block, one thread per node (FP32
+//                 sweeps and traces: per line): pointwise Euler flux (Eq. 2), sum-factorised
+//                 weak derivative along each direction, face lift, inverse mass (diagonal for
+//                 collocated Gauss points; folded into the tables), the low-storage RK update
+//                 (Eq. 10 or the 2N form), and the face traces of the next stage input.
 // or one kernel:
-//   vol_faces_kernel : the volume kernel with each element evaluating the numerical flux
+//   vol_faces_kernel(_fp64) : the volume kernel with each element evaluating the numerical flux
 //                 on its own faces from the stored traces (no face-flux array).
 // Index arithmetic is 32-bit: the host rejects meshes with 2^31 or more degrees of freedom.
 #pragma once
