@@ -16,6 +16,11 @@ constexpr int kMaxCoefDelay = 16;
 struct FixedScale {
   int eout, elo, ehi;
 };
+constexpr int kFixedValueBits = 61;  // bits of a fixed-point value below its exponent
+constexpr int kFixedMinExp = 61;     // smallest value exponent (the lowest bit stays normal)
+constexpr int kSweepFrac = 1, kTraceFrac = 2;  // fractional bits that a result keeps
+constexpr int fixed_out(int frac) { return 65 - frac; }  // eout plus the table's exponent
+constexpr long long fixed_half(int frac) { return 1ll << (30 - frac); }  // half of the last bit kept
 struct FixedTrace {  // rows l_a(-1) and l_a(+1), the limbs of an entry side by side
   int2 t[2][kMaxN];
   long long c[2];  // start values of the middle limb sums (fixline.cuh)
@@ -25,7 +30,7 @@ struct FixedTrace {  // rows l_a(-1) and l_a(+1), the limbs of an entry side by 
 struct FixedSweep {  // direction d, row i: N flux weights, low-face and high-face weight
   int2 q[3][kMaxN * (kMaxN + 2)];  // entry [i*(N+2) + k]
   long long c[3][kMaxN];           // start value of the middle limb sum per row (fixline.cuh)
-  FixedScale s;                    // one scale for all directions
+  FixedScale s[3];                 // per direction; elo and ehi are the same in all of them
 };
 
 // Operator tables in FP64; kernels convert entries to their arithmetic type.

@@ -107,9 +107,9 @@ struct FusedSmem {
   static constexpr size_t BIG = 2 * SLOT;
   static constexpr size_t FF = BIG + BIGB;
   static constexpr size_t BAR = FF + FFB;
-  static constexpr size_t MAXOFF = BAR + 16;  // largest magnitudes per element and variable (FP64)
+  static constexpr size_t EXPOFF = BAR + 16;  // exponents of the lines [EPB][D][NV][NF] (FP64)
   static constexpr size_t BYTES =
-      MAXOFF + (std::is_same<R, double>::value ? sizeof(int) * F::EPB * F::NV : 0);
+      EXPOFF + (std::is_same<R, double>::value ? sizeof(short) * F::EPB * D * F::NV * F::NF : 0);
 };
 
 // ---- TMA tensor copies (PTX; the mbarrier helpers are in kernels.cuh) -------------
@@ -178,7 +178,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
   R* sFF = reinterpret_cast<R*>(smem + SM::FF);
   float2* sFF2 = reinterpret_cast<float2*>(smem + SM::FF);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + SM::BAR);
-  int* sMax = reinterpret_cast<int*>(smem + SM::MAXOFF);
+  short* sExp = reinterpret_cast<short*>(smem + SM::EXPOFF);
 
   const VolArgs& V = A.v;
   const MeshArgs& m = V.m;
@@ -391,19 +391,15 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
     __syncthreads();
 
     // ---- B2. pointwise Euler fluxes (over U and T, both no longer needed) -----------------
-    // face ds = 2 d + side of this thread's element: low plane = its own tile coordinate
-    auto face_of = [=](int ds) {
-      const int d = ds >> 1;
-      const int lo = d == 0 ? (ez * TY + ey) * (TX + 1) + ex
-                            : (d == 1 ? F::F0 + (ez * (TY + 1) + ey) * TX + ex
-                                      : F::F0 + F::F1 + (ez * TY + ey) * TX + ex);
+    // face ds = 2 d + side of tile element te: low plane = its own tile coordinate
+    auto face_of = [](int te, int ds) {
+      const int d = ds >> 1, x = te % TX, y = (te / TX) % TY, z = te / (TX * TY);
+      const int lo = d == 0 ? (z * TY + y) * (TX + 1) + x
+                            : (d == 1 ? F::F0 + (z * (TY + 1) + y) * TX + x
+                                      : F::F0 + F::F1 + (z * TY + y) * TX + x);
       return (ds & 1) ? lo + (d == 0 ? 1 : (d == 1 ? TX : TX * TY)) : lo;
     };
-    // FP64: sweep tables, exponents per variable, FP64 chain needed
-    const FixedSweep* ftab = V.scaled ? &V.tab->fxs : &V.tab->fx;
-    const FixedScale fsc = ftab->s;
-    int fex[NV];
-    bool chain = false;
+    const FixedSweep* ftab = V.scaled ? &V.tab->fxs : &V.tab->fx;  // FP64
     {
       R Fp[D][NV];
       euler_flux_all<D, R>(u, Arith<R>::pair(V.gm1, V.gm1f), Fp);
@@ -414,37 +410,6 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
           for (int pr = 0; pr < NP; ++pr)
             sF2[((el * D + d) * NP + pr) * ND + node] =
                 make_float2(Fp[d][2 * pr], 2 * pr + 1 < NV ? Fp[d][2 * pr + 1] : 0.0f);
-      } else if constexpr (std::is_same<R, double>::value) {
-        // fixed point as in vol_body_fp64: per element and variable one exponent over the
-        // pointwise fluxes and the fluxes on the element's faces
-        for (int i = tid; i < EPB * NV; i += THREADS) sMax[i] = 0;
-        __syncthreads();
-        if (active) {
-#pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            int mx = abs_hi(Fp[0][v]);
-#pragma unroll
-            for (int d = 1; d < D; ++d) mx = max(mx, abs_hi(Fp[d][v]));
-            for (int q = node; q < 2 * D * NF; q += ND) {
-              const int ds = q / NF, j = q - ds * NF;
-              mx = max(mx, abs_hi(sFF[(face_of(ds) * NV + v) * NF + j]));
-            }
-            atomicMax(sMax + el * NV + v, mx);
-          }
-        }
-        __syncthreads();
-        if (active) {
-#pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            fex[v] = fixed_exponent(fsc, sMax[el * NV + v]);
-            chain = chain || fixed_outside(fsc, sMax[el * NV + v]);
-          }
-#pragma unroll
-          for (int d = 0; d < D; ++d)
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-              sF[((el * D + d) * NV + v) * ND + node] = chain ? Fp[d][v] : fixed_bits(Fp[d][v], fex[v] + kSweepShift);
-        }
       } else {
 #pragma unroll
         for (int d = 0; d < D; ++d)
@@ -453,6 +418,29 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
       }
     }
     __syncthreads();
+    if constexpr (std::is_same<R, double>::value) {
+      // fixed point line by line as in vol_body_fp64 (a face has another exponent in each of its
+      // two elements: its fluxes are converted where they are used)
+      for (int g = tid; g < EPB * D * NV * NF; g += THREADS) {
+        const int j = g % NF, dv = (g / NF) % (D * NV), te = g / (D * NV * NF);
+        const int v = dv % NV, d = dv / NV;
+        double* x = sF + (te * D * NV + dv) * ND + line_base<D, N>(d, j);
+        const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+        double val[N + 2];
+#pragma unroll
+        for (int a = 0; a < N; ++a) val[a] = x[a * stride];
+        val[N] = sFF[(face_of(te, 2 * d) * NV + v) * NF + j];
+        val[N + 1] = sFF[(face_of(te, 2 * d + 1) * NV + v) * NF + j];
+        int es;
+        const int lx = line_exponent<N>(val, ftab->s[d], es);
+        sExp[g] = (short)lx;
+        if (lx != kChainLine) {
+#pragma unroll
+          for (int a = 0; a < N; ++a) x[a * stride] = fixed_bits(val[a], es);
+        }
+      }
+      __syncthreads();
+    }
 
     // ---- D1. weak derivative + face lift ----------------------------------------------------
     using Acc = typename Arith<R>::Acc;
@@ -463,43 +451,49 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
       int flo[3], fhi[3];  // faces of this element along d
 #pragma unroll
       for (int d = 0; d < D; ++d) {
-        flo[d] = face_of(2 * d);
-        fhi[d] = face_of(2 * d + 1);
+        flo[d] = face_of(el, 2 * d);
+        fhi[d] = face_of(el, 2 * d + 1);
       }
-      bool fixed = false;
       if constexpr (std::is_same<R, double>::value) {
-        if (!chain) {
-          fixed = true;
-          FixedAcc fa[NV];
+        const short* xp[D];  // exponents of the node's lines
 #pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            long long c = 0;
+        for (int d = 0; d < D; ++d) xp[d] = sExp + (el * D + d) * NV * NF + face_index<D, N>(d, ix);
+        int xm[NV];
+        bool chain = false;
 #pragma unroll
-            for (int d = 0; d < D; ++d) c += ftab->c[d][ix[d]];
-            fa[v] = FixedAcc{0, fixed_start(fsc, fex[v], c)};
-          }
+        for (int v = 0; v < NV; ++v) {
+          xm[v] = xp[0][v * NF];
+#pragma unroll
+          for (int d = 1; d < D; ++d) xm[v] = max(xm[v], (int)xp[d][v * NF]);
+          chain = chain || xm[v] == kChainLine;
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          long long sum = 0;
 #pragma unroll
           for (int d = 0; d < D; ++d) {
-            const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
-            const int base = node - ix[d] * stride, j = face_index<D, N>(d, ix);
-            const int2* q = ftab->q[d] + ix[d] * (N + 2);
-#pragma unroll
-            for (int a = 0; a < N; ++a)
-#pragma unroll
-              for (int v = 0; v < NV; ++v)
-                fixed_fma(q[a], fixed_of_bits(sF[((el * D + d) * NV + v) * ND + base + a * stride]), fa[v]);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-              int2 flw = fixed_limbs(sFF[(flo[d] * NV + v) * NF + j], fex[v] + kSweepShift);
-              int2 fhw = fixed_limbs(sFF[(fhi[d] * NV + v) * NF + j], fex[v] + kSweepShift);
-              opaque(flw);
-              opaque(fhw);
-              fixed_fma(q[N], flw, fa[v]);
-              fixed_fma(q[N + 1], fhw, fa[v]);
+            const int stride = d == 0 ? 1 : (d == 1 ? N : N * N), j = face_index<D, N>(d, ix);
+            const double* x = sF + ((el * D + d) * NV + v) * ND + node - ix[d] * stride;
+            const double lo = sFF[(flo[d] * NV + v) * NF + j], hi = sFF[(fhi[d] * NV + v) * NF + j];
+            const int lx = xp[d][v * NF];
+            if (lx == kChainLine) {
+              acc[v] = chain_line<N>(*V.tab, V.scaled, d, ix[d], x, stride, lo, hi, acc[v]);
+              continue;
             }
-          }
+            const int2* q = ftab->q[d] + ix[d] * (N + 2);
+            FixedAcc t{0, ftab->c[d][ix[d]]};
 #pragma unroll
-          for (int v = 0; v < NV; ++v) acc[v] = fixed_result(fa[v], fsc, fex[v]);
+            for (int a = 0; a < N; ++a) fixed_fma(q[a], fixed_of_bits(x[a * stride]), t);
+            const int es = limbs_of_line(lx, ftab->s[d]);
+            int2 flw = fixed_limbs(lo, es), fhw = fixed_limbs(hi, es);
+            opaque(flw);
+            opaque(fhw);
+            fixed_fma(q[N], flw, t);
+            fixed_fma(q[N + 1], fhw, t);
+            if (chain) acc[v] += line_result(fixed_sum<kSweepFrac>(t), lx);
+            else add_line(t, lx, xm[v], sum);
+          }
+          if (!chain) acc[v] = line_result(sum, xm[v]);
         }
       }
       if constexpr (PK) {
@@ -536,7 +530,7 @@ fused_kernel(const __grid_constant__ FusedArgs A, const __grid_constant__ CUtens
 #pragma unroll
           for (int v = 0; v < NV; ++v) acc[v] = (v & 1) ? a2[v / 2].y : a2[v / 2].x;
         }
-      } else if (!fixed) {
+      } else if constexpr (!std::is_same<R, double>::value) {
 #pragma unroll
         for (int d = 0; d < D; ++d) {
           const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);

@@ -115,7 +115,7 @@ void lagrange_at(int n, const long double* x, const long double* lam, long doubl
 }
 
 // ---- fixed-point tables of the FP64 contractions (fixline.cuh) ------------------------
-constexpr int kFixedSumBits = 61;  // bound of a contraction's sum of |entries|, in bits
+constexpr int kFixedSumBits = 61;  // bound of a line's sum of |entries|, in bits
 
 // limbs of a fixed-point table entry: v = x 2^31 + y, |y| <= 2^30
 int2 fixed_entry(int64_t v) {
@@ -123,14 +123,24 @@ int2 fixed_entry(int64_t v) {
   return make_int2((int)hi, (int)(v - hi * ((int64_t)1 << 31)));
 }
 
-// Exponents for a table stored as value 2^sq whose 64-bit results are value 2^-eout of the
-// values' exponent: results have to be normal numbers.
+// Exponents for a table whose 64-bit results are value 2^-eout of the values' exponent: results
+// have to be normal numbers, and so have the lowest bits of the values.
 FixedScale fixed_scale(int eout) {
   FixedScale f;
   f.eout = eout;
-  f.elo = eout < 4 ? 64 - eout : 60;
-  f.ehi = eout > -1 ? 2045 - eout : 2046;
+  f.elo = std::max(kFixedMinExp, 64 - eout);
+  f.ehi = std::min(2046, 2045 - eout);
   return f;
+}
+
+// Whether the middle limb sum of a row, sum |q1| 2^31 + |q0| 2^(kFixedValueBits - 31), stays
+// below 2^63.
+bool fixed_row_fits(const int2* q, int n) {
+  unsigned __int128 sum = (unsigned __int128)1 << 34;  // more than the start value
+  for (int k = 0; k < n; ++k)
+    sum += ((unsigned __int128)std::llabs(q[k].x) << 31) +
+           ((unsigned __int128)std::llabs(q[k].y) << (kFixedValueBits - 31));
+  return sum >> 63 == 0;
 }
 
 // largest row sum of |v| of a rows x cols table
@@ -153,42 +163,41 @@ int fixed_shift(long double sum) {
 }
 
 // Sweep tables times dt (scaled) or as they are, from the integers of build_tables: an integer
-// product with the mantissa of dt.  One scale for all directions, whose sum a contraction
-// forms; entries are halved once more where the middle limb sum of the worst row,
-// sum |q1| 2^31 + |q0| 2^28, could reach 2^63.
+// product with the mantissa of dt.  Every direction has a scale of its own, so that the entries
+// of the longer sides of a stretched element keep all their bits; entries are halved once more
+// where a row's middle limb sum could overflow.
 void fixed_sweep_tables(const adg_solver* s, double dt, bool scaled, FixedSweep* f) {
   const int N = s->N, M = N + 2;
-  int ex = 0;
+  int ex = 0, elo = 0, ehi = 2046;
   const int64_t mant = scaled ? (int64_t)std::ldexp(std::frexp(dt, &ex), 53) : 0;  // dt = mant 2^(ex-53)
-  int sh = 0;
-  if (scaled) {
-    __int128 sum = 0;
-    for (int d = 0; d < s->dim; ++d) sum += (__int128)row_sum_max(s->fix_q[d], N, M) * mant;
-    sh = (sum >> 52) <= ((__int128)1 << kFixedSumBits) ? 52 : 53;
-  }
-  for (;; ++sh) {
-    unsigned __int128 worst = 0;
-    for (int d = 0; d < s->dim; ++d) {
-      unsigned __int128 big = 0;
+  for (int d = 0; d < s->dim; ++d) {
+    int sh = 0;
+    if (scaled) {
+      const __int128 sum = (__int128)row_sum_max(s->fix_q[d], N, M) * mant;
+      sh = (sum >> 52) <= ((__int128)1 << kFixedSumBits) ? 52 : 53;
+    }
+    for (bool fits = false; !fits; ++sh) {
+      fits = true;
       for (int i = 0; i < N; ++i) {
-        unsigned __int128 sum = 0;
-        f->c[d][i] = d == 0 ? (long long)1 << 30 : 0;
+        int2* row = &f->q[d][i * M];
+        f->c[d][i] = fixed_half(kSweepFrac);
         for (int k = 0; k < M; ++k) {
           const __int128 v = (__int128)s->fix_q[d][i * M + k] * (scaled ? mant : 1);
-          const int2 q = fixed_entry((int64_t)(sh > 0 ? (v + ((__int128)1 << (sh - 1))) >> sh : v));
-          f->q[d][i * M + k] = q;
-          f->c[d][i] += q.y / 2;
-          sum += ((unsigned __int128)(q.x < 0 ? -(int64_t)q.x : q.x) << 31) +
-                 ((unsigned __int128)(q.y < 0 ? -(int64_t)q.y : q.y) << 28);
+          row[k] = fixed_entry((int64_t)(sh > 0 ? (v + ((__int128)1 << (sh - 1))) >> sh : v));
+          f->c[d][i] += row[k].y / 2;
         }
-        big = sum > big ? sum : big;
+        fits = fits && fixed_row_fits(row, M);
       }
-      worst += big;
+      // value 2^sq with sq = fix_s + 53 - sh - ex (scaled) or fix_s - sh
+      f->s[d] = fixed_scale(fixed_out(kSweepFrac) - (scaled ? s->fix_s[d] + 53 - sh - ex : s->fix_s[d] - sh));
     }
-    if (worst >> 63 == 0) break;
+    elo = std::max(elo, f->s[d].elo);
+    ehi = std::min(ehi, f->s[d].ehi);
   }
-  // value 2^sq with sq = fix_s + 53 - sh - ex (scaled) or fix_s - sh
-  f->s = fixed_scale(67 - (scaled ? s->fix_s + 53 - sh - ex : s->fix_s - sh));
+  for (int d = 0; d < s->dim; ++d) {
+    f->s[d].elo = elo;
+    f->s[d].ehi = ehi;
+  }
 }
 
 // packed FP32 sweep table from the FP32-pair one
@@ -250,20 +259,18 @@ void build_tables(adg_solver* s) {
   // the same rows in fixed point: per direction N flux weights, low and high face
   {
     const int M = N + 2;
-    long double rows[3][kMaxN * (kMaxN + 2)], sum = 0.0L;
+    long double rows[kMaxN * (kMaxN + 2)];
     for (int d = 0; d < s->dim; ++d) {
       const long double sc = 2.0L / (long double)s->h[d];
       for (int i = 0; i < N; ++i) {
         for (int a = 0; a < N; ++a)
-          rows[d][i * M + a] = sc * (long double)wd[a] * Dm[a][i] / (long double)wd[i];
-        rows[d][i * M + N] = 0.5L * sc * lm[i] / (long double)wd[i];
-        rows[d][i * M + N + 1] = -0.5L * sc * lp[i] / (long double)wd[i];
+          rows[i * M + a] = sc * (long double)wd[a] * Dm[a][i] / (long double)wd[i];
+        rows[i * M + N] = 0.5L * sc * lm[i] / (long double)wd[i];
+        rows[i * M + N + 1] = -0.5L * sc * lp[i] / (long double)wd[i];
       }
-      sum += row_sum_max(rows[d], N, M);
+      s->fix_s[d] = fixed_shift(row_sum_max(rows, N, M));
+      for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[i], s->fix_s[d]));
     }
-    s->fix_s = fixed_shift(sum);
-    for (int d = 0; d < s->dim; ++d)
-      for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[d][i], s->fix_s));
     fixed_sweep_tables(s, 0.0, false, &T.fx);
     const int st = fixed_shift(std::max(row_sum_max(lm, 1, N), row_sum_max(lp, 1, N)));
     for (int a = 0; a < N; ++a) {
@@ -274,10 +281,10 @@ void build_tables(adg_solver* s) {
     }
     for (int d = 0; d < s->dim; ++d) packed_table(N, T.Qf[d], T.qp[d]);
     for (int side = 0; side < 2; ++side) {
-      T.ft.c[side] = (long long)1 << 30;
+      T.ft.c[side] = fixed_half(kTraceFrac);
       for (int a = 0; a < N; ++a) T.ft.c[side] += T.ft.t[side][a].y / 2;
     }
-    T.ft.s = fixed_scale(66 - st);
+    T.ft.s = fixed_scale(fixed_out(kTraceFrac) - st);
   }
   double xe[16], we[16];
   gauss_legendre(N + 1, xe, we);

@@ -1101,43 +1101,6 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, const SweepArg<D, N, 
 
 // ---- FP64 volume/update work --------------------------------------------------------
 
-// Elements that a warp of a tile of THREADS nodes touches, at most.
-template <int ND, int THREADS>
-constexpr int warp_elements() {
-  int most = 1;
-  for (int w = 0; w < THREADS; w += 32) {
-    const int end = (w + 31 < THREADS ? w + 31 : THREADS - 1) / ND - w / ND + 1;
-    most = end > most ? end : most;
-  }
-  return most;
-}
-
-// Maximum of m over the lanes of each element (el: this lane's element, -1: none) into
-// smax[el * NV + v]; lanes of one element are neighbours.
-template <int ND, int NV, int THREADS>
-__device__ __forceinline__ void element_max(const int (&m)[NV], int el, int* smax) {
-  if constexpr (ND < 16) {
-    if (el >= 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) atomicMax(smax + el * NV + v, m[v]);
-    }
-  } else {
-    // one warp reduction per element the warp touches, then one atomic per variable
-    const int lane = threadIdx.x & 31, first = (int)(threadIdx.x - lane) / ND;
-#pragma unroll
-    for (int k = 0; k < warp_elements<ND, THREADS>(); ++k) {
-      const bool in = el == first + k;
-      int mine = 0;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const int r = __reduce_max_sync(0xFFFFFFFFu, in ? m[v] : 0);
-        if (lane == v) mine = r;
-      }
-      if (lane < NV && mine > 0) atomicMax(smax + (first + k) * NV + lane, mine);
-    }
-  }
-}
-
 // Limbs of a value in its place.
 __device__ __forceinline__ double fixed_bits(double x, int es) {
   const int2 f = fixed_limbs(x, es);
@@ -1147,10 +1110,26 @@ __device__ __forceinline__ int2 fixed_of_bits(double b) {
   return make_int2(__double2hiint(b), __double2loint(b));
 }
 
+// Row i of direction d over a line in FP64: k + the sweep over x (a line of nodes with a stride)
+// and the lift of its two face fluxes.
+template <int N>
+__device__ __forceinline__ double chain_line(const OpTables& tab, int scaled, int d, int i, const double* x,
+                                             int stride, double lo, double hi, double k) {
+  const double* q = (scaled ? tab.Qs[d] : tab.Q[d]) + i * N;
+#pragma unroll 1
+  for (int a = 0; a < N; ++a) k = fma(q[a], x[a * stride], k);
+  k = fma((scaled ? tab.Lms[d] : tab.Lm[d])[i], lo, k);
+  return fma(-(scaled ? tab.Lps[d] : tab.Lp[d])[i], hi, k);
+}
+
 // Shared memory of the FP64 volume kernel: pointwise fluxes [D][NV][THREADS] and face fluxes
 // [EPB][D][side][NV][NF] (as limbs, or FP64 for the FP64 chain), the staged solution and
 // Runge-Kutta register [NV][THREADS] (the solution's place then takes the next stage input),
-// the fixed-point sweep tables, and the largest magnitudes per element and variable.
+// the fixed-point sweep tables, and the exponents of every line of nodes [D][EPB * NF].
+template <int D>
+struct __align__(D == 2 ? 8 : 16) LineExp {  // one per variable, two in a word
+  unsigned w[D == 2 ? 2 : 4];
+};
 template <int D, int N, int TT>
 struct VolSmem64 {
   using T = Tile<D, N, TT>;
@@ -1160,22 +1139,24 @@ struct VolSmem64 {
   static constexpr size_t Q_OFF = W_OFF + sizeof(double) * T::NV * T::THREADS;
   static constexpr size_t TAB_OFF = Q_OFF + sizeof(double) * T::NV * T::THREADS;
   static constexpr size_t C_OFF = TAB_OFF + sizeof(int2) * D * N * (N + 2);
-  static constexpr size_t MAX_OFF = C_OFF + sizeof(long long) * D * N;
-  static constexpr size_t BYTES = MAX_OFF + sizeof(int) * T::EPB * T::NV;
+  static constexpr size_t EXP_OFF = (C_OFF + sizeof(long long) * D * N + 15) / 16 * 16;
+  static constexpr size_t BYTES = EXP_OFF + sizeof(LineExp<D>) * D * T::EPB * T::NF;
 };
 
 // One element tile of the FP64 volume/update kernel.  Everything the tile reads is copied to
 // shared memory asynchronously at the start; one thread per node evaluates the pointwise
-// fluxes, the sweeps with the lift (in fixed point, fixline.cuh) and the Runge-Kutta update;
-// one thread per line interpolates the traces of the next stage input.
-// Bound: the FP64 pipe retires 2 operations per clock and SM (and each takes about five issue
-// slots), so whatever is a contraction runs on the integer pipe (2D p=4: 23 FP64 operations
-// per node instead of 97); the pointwise fluxes and the update stay in FP64.  FP64 pipe 56 %,
-// ALU 56 %, issue 68 % busy.  Against chains of FP64 fused multiply-adds: 256^2 p=4 295 -> 112
-// us, 320^2 p=3 265 -> 102, 160^2 p=7 349 -> 112, 48^3 p=3 1874 -> 670, 32^3 p=5 2291 -> 850.
-// One exponent per element and variable (each value is converted once and the directions add
-// up as integers) against one per line of nodes with a thread per line: 256^2 112 against 135
-// us, 48^3 670 against 904.
+// fluxes, one per line of nodes turns them and the face fluxes into fixed point, one per node
+// forms the sweeps with the lift (fixline.cuh) and the Runge-Kutta update; one thread per line
+// interpolates the traces of the next stage input.
+// Bound: the FP64 pipe retires 2 operations per clock and SM, so whatever is a contraction runs
+// on the integer pipe (2D p=4: 23 FP64 operations per node instead of 97); the pointwise fluxes
+// and the update stay in FP64.  Against chains of FP64 fused multiply-adds: 256^2 p=4 295 -> 117
+// us, 320^2 p=3 265 -> 107, 160^2 p=7 349 -> 117, 48^3 p=3 1874 -> 760, 32^3 p=5 2291 -> 880.
+// Every line of nodes has an exponent of its own and every direction a table scale of its own,
+// as a node's error has to be that of the lines through it.  (One exponent per element and
+// variable and one scale for all directions: 48^3 687 us, 256^2 114 us, but a node whose lines
+// are 10^-6 of the element's largest value was wrong from the eleventh digit on, and so was the
+// flow along the sides of an element 10^6 times as long as wide.)
 template <int D, int N, int TT, typename Faces = SplitFaces>
 __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsigned char* smem_raw,
                                               const Faces& faces = Faces()) {
@@ -1183,7 +1164,7 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
   constexpr bool kFaces = std::is_same<Faces, ElementFaces>::value;
   using SM = VolSmem64<D, N, TT>;
   constexpr int ND = T::ND, NF = T::NF, NV = T::NV, EPB = T::EPB, M = N + 2;
-  constexpr int THREADS = T::THREADS, BLOCK = SM::BLOCK;
+  constexpr int THREADS = T::THREADS, BLOCK = SM::BLOCK, LINES = EPB * NF;
   const int tid = threadIdx.x;
   double* sF = reinterpret_cast<double*>(smem_raw);
   double* sFace = reinterpret_cast<double*>(smem_raw + SM::FACE_OFF);
@@ -1191,7 +1172,7 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
   double* sQ = reinterpret_cast<double*>(smem_raw + SM::Q_OFF) + tid;
   int2* sTab = reinterpret_cast<int2*>(smem_raw + SM::TAB_OFF);  // [D][N][M]
   long long* sC = reinterpret_cast<long long*>(smem_raw + SM::C_OFF);  // [D][N]
-  int* sMax = reinterpret_cast<int*>(smem_raw + SM::MAX_OFF);    // [EPB][NV]
+  LineExp<D>* sExp = reinterpret_cast<LineExp<D>*>(smem_raw + SM::EXP_OFF);  // [D][LINES]
   const int el = tid / ND, node = tid - el * ND;
   const int e0 = tile * EPB;
   const int ne = (int)A.m.ne;
@@ -1237,133 +1218,143 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
   for (int i = tid; i < D * N * M; i += BLOCK) cp_async8(sTab + i, &tab->q[i / (N * M)][i % (N * M)]);
   if (tid < D * N) cp_async8(sC + tid, &tab->c[tid / N][tid % N]);
   cp_async_commit();
-  for (int i = tid; i < EPB * NV; i += BLOCK) sMax[i] = 0;
-  __syncthreads();
 
-  // 1. pointwise fluxes; largest magnitude of every variable's fluxes in the element
+  // 1. pointwise fluxes
   cp_async_wait<1>();
-  double F[D][NV];
-  {
-    double u[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) u[v] = active ? (from_r ? sQ : sW)[v * THREADS] : 1.0;
-    euler_flux_all<D, double>(u, A.gm1, F);
-  }
-  cp_async_wait<0>();
-  {
-    int m[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      m[v] = abs_hi(F[0][v]);
-#pragma unroll
-      for (int d = 1; d < D; ++d) m[v] = max(m[v], abs_hi(F[d][v]));
-    }
-    if (active) {
-      for (int q = node; q < 2 * D * NF; q += ND) {
-        const int ds = q / NF, j = q - ds * NF;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-          m[v] = max(m[v], abs_hi(sFace[((el * 2 * D + ds) * NV + v) * NF + j]));
-      }
-    }
-    element_max<ND, NV, THREADS>(m, active ? el : -1, sMax);
-  }
-  __syncthreads();
-
-  // 2. fixed point (or the values as they are where the element needs the FP64 chain)
-  int ex[NV];
-  bool chain = false;
-  const FixedScale sc = tab->s;
   if (active) {
+    double F[D][NV], u[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int mx = sMax[el * NV + v];
-      ex[v] = fixed_exponent(sc, mx);
-      chain = chain || fixed_outside(sc, mx);
-    }
-    if (!chain) {
-#pragma unroll
-      for (int d = 0; d < D; ++d)
-#pragma unroll
-        for (int v = 0; v < NV; ++v) F[d][v] = fixed_bits(F[d][v], ex[v] + kSweepShift);
-      for (int q = node; q < 2 * D * NF; q += ND) {
-        const int ds = q / NF, j = q - ds * NF;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          double* f = sFace + ((el * 2 * D + ds) * NV + v) * NF + j;
-          *f = fixed_bits(*f, ex[v] + kSweepShift);
-        }
-      }
-    }
+    for (int v = 0; v < NV; ++v) u[v] = (from_r ? sQ : sW)[v * THREADS];
+    euler_flux_all<D, double>(u, A.gm1, F);
 #pragma unroll
     for (int d = 0; d < D; ++d)
 #pragma unroll
       for (int v = 0; v < NV; ++v) sF[(d * NV + v) * THREADS + tid] = F[d][v];
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+
+  // 2. fixed point, one thread per line of nodes with its two face fluxes: a thread takes the
+  // same line of several (direction, variable) pairs.  With an even number of nodes their order
+  // does not matter here: where it is a power of two, lines that start in the same bank are
+  // walked in different orders (without: 320^2 p=3 114 against 109 us, 160^2 p=7 125 against 116,
+  // 48^3 p=3 797 against 783).  Two pairs at a time: 48^3 774 against 775, 40^3 p=4 896 against
+  // 906 us; four: 807 and 903.
+  {
+    constexpr int GROUPS = BLOCK / LINES;
+    constexpr bool kPow2 = (N & (N - 1)) == 0;
+    const int r = tid % LINES, le = r / NF, j = r - le * NF;  // r = el * NF + j
+    FixedScale sc = tab->s[0];
+    const int eout[3] = {sc.eout, tab->s[1].eout, tab->s[2].eout};
+    if (tid < GROUPS * LINES && e0 + le < ne) {
+#pragma unroll 2
+      for (int dv = tid / LINES; dv < D * NV; dv += GROUPS) {
+        const int d = dv / NV, v = dv - d * NV;
+        int st, es;
+        const int base = tile_line<D, N, N>(d, r, st);
+        const int turn = kPow2 ? ((base >> 4) + (base >> 6)) & (N - 1) : 0;
+        double* x = sF + dv * THREADS + base;
+        double* f = sFace + ((le * D + d) * 2 * NV + v) * NF + j;
+        double val[M];
+#pragma unroll
+        for (int a = 0; a < N; ++a) val[a] = x[(a ^ turn) * st];
+        val[N] = f[0];
+        val[N + 1] = f[NV * NF];
+        sc.eout = d == 0 ? eout[0] : (d == 1 ? eout[1] : eout[2]);
+        const int ex = line_exponent<N>(val, sc, es);
+        unsigned short* out = reinterpret_cast<unsigned short*>(sExp[d * LINES + r].w) + v;
+        if (D == 3 && v == NV - 1) *reinterpret_cast<unsigned*>(out) = (unsigned)ex;
+        else *out = (unsigned short)ex;
+        if (ex != kChainLine) {
+#pragma unroll
+          for (int a = 0; a < N; ++a) x[(a ^ turn) * st] = fixed_bits(val[a], es);
+          f[0] = fixed_bits(val[N], es);
+          f[NV * NF] = fixed_bits(val[N + 1], es);
+        }
+      }
+    }
   }
   __syncthreads();
 
   // 3. weak derivative (one contraction per direction) and face lift, Runge-Kutta update
   if (active) {
     const int ix[3] = {node % N, (node / N) % N, node / (N * N)};
-    double k[NV];
+    constexpr int NW = (NV + 1) / 2;
+    unsigned lx[D][NW], any = 0;  // exponents of the node's lines
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const LineExp<D> q = sExp[d * LINES + el * NF + face_index<D, N>(d, ix)];
+#pragma unroll
+      for (int w = 0; w < NW; ++w) any |= lx[d][w] = q.w[w];
+    }
+    auto line_ex = [&](int d, int v) { return (int)((lx[d][v >> 1] >> (16 * (v & 1))) & 0xFFFF); };
+    const bool chain = any & (kChainLine * 0x10001u);
     if (!chain) {
-      FixedAcc acc[NV];
-      long long c = sC[ix[0]];
+      long long sum[NV];
+      int ex[NV];
 #pragma unroll
-      for (int d = 1; d < D; ++d) c += sC[d * N + ix[d]];
+      for (int v = 0; v < NV; ++v) {
+        sum[v] = 0;
+        ex[v] = line_ex(0, v);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] = FixedAcc{0, fixed_start(sc, ex[v], c)};
+        for (int d = 1; d < D; ++d) ex[v] = max(ex[v], line_ex(d, v));
+      }
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
         const double* f = sF + d * NV * THREADS + tid - ix[d] * stride;
+        const double* g = sFace + (el * D + d) * 2 * NV * NF + face_index<D, N>(d, ix);
         const int2* q = sTab + (d * N + ix[d]) * M;
+        const long long c = sC[d * N + ix[d]];
+        FixedAcc acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = FixedAcc{0, c};
 #pragma unroll
         for (int a = 0; a < N; ++a) {
           const int2 w = q[a];
 #pragma unroll
           for (int v = 0; v < NV; ++v) fixed_fma(w, fixed_of_bits(f[v * THREADS + a * stride]), acc[v]);
         }
-        const double* g = sFace + (el * D + d) * 2 * NV * NF + face_index<D, N>(d, ix);
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
           const int2 w = q[N + side];
 #pragma unroll
           for (int v = 0; v < NV; ++v) fixed_fma(w, fixed_of_bits(g[(side * NV + v) * NF]), acc[v]);
         }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) add_line(acc[v], line_ex(d, v), ex[v], sum[v]);
       }
 #pragma unroll
-      for (int v = 0; v < NV; ++v) k[v] = fixed_result(acc[v], sc, ex[v]);
-    } else {
-      const double* sFv = sF + tid;
+      for (int v = 0; v < NV; ++v)
+        sW[v * THREADS] = Update<double>::apply(A, (v * ne + e) * ND + node, line_result(sum[v], ex[v]),
+                                                sW[v * THREADS], sQ[v * THREADS]);
+    } else {  // line by line
+#pragma unroll 1
+      for (int v = 0; v < NV; ++v) {
+        double k = 0.0;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) k[v] = 0.0;
-      for (int pass = 0; pass < 2 * D; ++pass) {  // the sweeps, then the lifts
-        const int d = pass < D ? pass : pass - D;
-        const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
-        const int id = d == 0 ? ix[0] : (d == 1 ? ix[1] : ix[2]);
-        if (pass < D) {
-          const double* f = sFv + d * NV * THREADS - id * stride;
-          const double* Q = (A.scaled ? A.tab->Qs[d] : A.tab->Q[d]) + id * N;
-          for (int a = 0; a < N; ++a)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) k[v] = fma(Q[a], f[v * THREADS + a * stride], k[v]);
-        } else {
-          const double lm = (A.scaled ? A.tab->Lms[d] : A.tab->Lm[d])[id];
-          const double lp = (A.scaled ? A.tab->Lps[d] : A.tab->Lp[d])[id];
-          const double* g = sFace + (el * D + d) * 2 * NV * NF + face_index<D, N>(d, ix);
-#pragma unroll
-          for (int v = 0; v < NV; ++v) {
-            k[v] = fma(lm, g[v * NF], k[v]);
-            k[v] = fma(-lp, g[(NV + v) * NF], k[v]);
+        for (int d = 0; d < D; ++d) {
+          const int stride = d == 0 ? 1 : (d == 1 ? N : N * N);
+          const double* f = sF + (d * NV + v) * THREADS + tid - ix[d] * stride;
+          const double* g = sFace + ((el * D + d) * 2 * NV + v) * NF + face_index<D, N>(d, ix);
+          const int ex = reinterpret_cast<const unsigned short*>(
+              sExp[d * LINES + el * NF + face_index<D, N>(d, ix)].w)[v];
+          if (ex == kChainLine) {
+            k = chain_line<N>(*A.tab, A.scaled, d, ix[d], f, stride, g[0], g[NV * NF], k);
+          } else {
+            const int2* q = sTab + (d * N + ix[d]) * M;
+            FixedAcc acc{0, sC[d * N + ix[d]]};
+#pragma unroll 1
+            for (int a = 0; a < N; ++a) fixed_fma(q[a], fixed_of_bits(f[a * stride]), acc);
+            fixed_fma(q[N], fixed_of_bits(g[0]), acc);
+            fixed_fma(q[N + 1], fixed_of_bits(g[NV * NF]), acc);
+            k += line_result(fixed_sum<kSweepFrac>(acc), ex);
           }
         }
+        sW[v * THREADS] = Update<double>::apply(A, (v * ne + e) * ND + node, k, sW[v * THREADS],
+                                                sQ[v * THREADS]);
       }
     }
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-      sW[v * THREADS] = Update<double>::apply(A, (v * ne + e) * ND + node, k[v], sW[v * THREADS],
-                                              sQ[v * THREADS]);
   }
 
   // 4. traces of the next stage input
@@ -1381,8 +1372,10 @@ template <int D, int N, typename R> struct VolKernelRegs {
   static constexpr int value = (D == 2 && (N == 2 || N == 8)) ? 64 : 56;  // no spills (ptxas)
 };
 template <int D, int N> struct VolKernelRegs<D, N, double> {
-  // 2D 40 to 64 registers within 2 %; 3D 48 registers spill (+5 %), 72 gain nothing
-  static constexpr int value = D == 2 ? 48 : 64;
+  // us at 48, 56, 64 registers: 256^2 p=4 118.0, 117.3, 118.4; 640^2 p=1 151, 143, 141; 160^2 p=7
+  // 116, 117, 121.  At 64, 72, 80: 48^3 p=3 783, 774, 759; 64^3 p=2 984, 923, 917; 32^3 p=5 889,
+  // 894, 939, but at 56 875.
+  static constexpr int value = D == 2 ? 56 : (N == 6 ? 56 : 80);
 };
 template <int D, int N> struct VolKernelRegs<D, N, float> {
   // 2D: 40 registers are 1 to 4 % slower (N = 8: 1 % faster); 3D: 32 spill (2 to 4 % slower),

@@ -43,8 +43,8 @@ struct adg_solver {
   double* tmp_k = nullptr;
   int red_blocks = 0;
   adg::OpTables tab{};
-  int64_t fix_q[3][adg::kMaxN * (adg::kMaxN + 2)] = {};  // unscaled sweep rows, q 2^fix_s
-  int fix_s = 0;
+  int64_t fix_q[3][adg::kMaxN * (adg::kMaxN + 2)] = {};  // unscaled sweep rows, q 2^fix_s[d]
+  int fix_s[3] = {};
   adg::MeshArgs margs{};
   int64_t npe = 0;
   int depth = 0, head = -1, n_iface = 0;
