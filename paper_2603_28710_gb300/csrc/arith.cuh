@@ -103,11 +103,14 @@ __device__ __forceinline__ float r_sqrt(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// Half the square root, FP64: an FP32 seed y0 of 1/sqrt(m) for the argument scaled to
-// m = s 2^(-2k) in [1, 4) (relative error about 2^-22), g = m y0 and e = 1 - g y0, then the
-// binomial series sqrt(m) = g (1 - e)^(-1/2) = g (1 + e/2 + 3 e^2/8 + ...) to second order
-// (the next term is below 2^-66): 5 FP64 operations instead of the IEEE sequence (about 20),
-// within 0.8 ulp.  Zero, subnormal, negative and non-finite arguments take sqrt().
+// Half the square root, FP64, rounded as the IEEE square root except with a chance of about
+// 2^-33: an FP32 seed y of 1/sqrt(m) for the argument scaled to m = s 2^(-2k) in [1, 4) (relative
+// error about 2^-22), one coupled Newton step for sqrt(m) and 1/(2 sqrt(m)) (Goldschmidt's
+// iteration; both to about 2^-43), then the correction g + (m - g^2) / (2 sqrt(m)) with the exact
+// residual (error 2^-86 before the last rounding): 6 FP64 operations instead of the IEEE
+// sequence's about 20.  (Without the step for 1/(2 sqrt(m)), 5 operations: 2^-13 of the results
+// rounded the other way; a binomial series in 5: errors up to 0.8 ulp.)  Zero, subnormal,
+// negative and non-finite arguments take sqrt().
 __device__ __forceinline__ double half_sqrt(double s) {
   const int hi = __double2hiint(s);
   if ((unsigned)(hi - 0x00100000) >= 0x7FE00000u) return 0.5 * sqrt(s);
@@ -116,8 +119,10 @@ __device__ __forceinline__ double half_sqrt(double s) {
   float y0;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(d2f_int(m)));
   const double y = f2d_int(y0), g = m * y;
-  const double e = fma(-g, y, 1.0);
-  const double r = fma(g * e, fma(e, 0.375, 0.5), g);
+  const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));  // y / 2
+  const double e = fma(-g, h, 0.5);
+  const double g1 = fma(g, e, g), h1 = fma(h, e, h);
+  const double r = fma(fma(-g1, g1, m), h1, g1);
   return __hiloint2double(__double2hiint(r) + (k2 >> 1) - 0x00100000, __double2loint(r));
 }
 // Larger of two squared speeds by integer comparison (the FP64 comparison would take the FP64

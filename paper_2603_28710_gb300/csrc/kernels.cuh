@@ -141,10 +141,10 @@ __device__ __forceinline__ void llf_flux(const R (&wm)[D + 2], const R (&wp)[D +
                                          R gamma, R gm1, R (&f)[D + 2]) {
   constexpr int NV = D + 2;
   if constexpr (std::is_same<R, double>::value) {
-    // Bound by the FP64 pipe, 2D 45 and 3D 53 operations (from about 78 and 81): the square
-    // root takes 5, the larger speed is found by integer comparison, and the two sides'
-    // products are summed as they are formed.  256^2 p=4: 81 -> 68 us per launch; 48^3 p=3:
-    // 677 -> 552 us.
+    // Bound by the FP64 pipe, 2D 46 and 3D 54 operations (from about 78 and 81): the square
+    // root takes 6, the larger speed is found by integer comparison, and the two sides'
+    // products are summed as they are formed.  256^2 p=4: 81 -> 69 us per launch; 48^3 p=3:
+    // 677 -> 558 us.
     double um, up, pm, pp, sm, sp;
     side_state<D, double>(wm, d, gamma, gm1, um, pm, sm);
     side_state<D, double>(wp, d, gamma, gm1, up, pp, sp);
