@@ -12,7 +12,8 @@ constexpr int kMaxRing = 24;    // ring levels (random_delay_max + np + 1 <= 15 
 constexpr int kMaxCoefDelay = 16;
 
 // Fixed-point operator tables of the FP64 contractions (fixline.cuh).  eout: exponent of a
-// result relative to that of its values; elo, ehi: value exponents the tables cover.
+// result relative to that of its values; elo, ehi: value exponents the tables cover (none if
+// ehi < 0).
 struct FixedScale {
   int eout, elo, ehi;
 };

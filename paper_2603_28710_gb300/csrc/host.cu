@@ -165,11 +165,14 @@ int fixed_shift(long double sum) {
 // Sweep tables times dt (scaled) or as they are, from the integers of build_tables: an integer
 // product with the mantissa of dt.  Every direction has a scale of its own, so that the entries
 // of the longer sides of a stretched element keep all their bits; entries are halved once more
-// where a row's middle limb sum could overflow.
+// where a row's middle limb sum could overflow.  A time step or an operator that is not finite has
+// no fixed-point form: the empty exponent range sends every line to the FP64 chains, whose tables
+// then give the non-finite results.
 void fixed_sweep_tables(const adg_solver* s, double dt, bool scaled, FixedSweep* f) {
   const int N = s->N, M = N + 2;
   int ex = 0, elo = 0, ehi = 2046;
-  const int64_t mant = scaled ? (int64_t)std::ldexp(std::frexp(dt, &ex), 53) : 0;  // dt = mant 2^(ex-53)
+  const bool usable = s->fix_ok && (!scaled || std::isfinite(dt));
+  const int64_t mant = scaled && usable ? (int64_t)std::ldexp(std::frexp(dt, &ex), 53) : 0;  // dt = mant 2^(ex-53)
   for (int d = 0; d < s->dim; ++d) {
     int sh = 0;
     if (scaled) {
@@ -196,7 +199,7 @@ void fixed_sweep_tables(const adg_solver* s, double dt, bool scaled, FixedSweep*
   }
   for (int d = 0; d < s->dim; ++d) {
     f->s[d].elo = elo;
-    f->s[d].ehi = ehi;
+    f->s[d].ehi = usable ? ehi : -1;
   }
 }
 
@@ -268,7 +271,12 @@ void build_tables(adg_solver* s) {
         rows[i * M + N] = 0.5L * sc * lm[i] / (long double)wd[i];
         rows[i * M + N + 1] = -0.5L * sc * lp[i] / (long double)wd[i];
       }
-      s->fix_s[d] = fixed_shift(row_sum_max(rows, N, M));
+      const long double sum = row_sum_max(rows, N, M);
+      if (!std::isfinite(sum)) {
+        s->fix_ok = false;
+        continue;
+      }
+      s->fix_s[d] = fixed_shift(sum);
       for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[i], s->fix_s[d]));
     }
     fixed_sweep_tables(s, 0.0, false, &T.fx);

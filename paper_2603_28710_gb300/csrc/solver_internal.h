@@ -45,6 +45,7 @@ struct adg_solver {
   adg::OpTables tab{};
   int64_t fix_q[3][adg::kMaxN * (adg::kMaxN + 2)] = {};  // unscaled sweep rows, q 2^fix_s[d]
   int fix_s[3] = {};
+  bool fix_ok = true;  // false: an entry of the operator is not finite
   adg::MeshArgs margs{};
   int64_t npe = 0;
   int depth = 0, head = -1, n_iface = 0;
