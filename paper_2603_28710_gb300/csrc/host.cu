@@ -369,6 +369,13 @@ uint64_t splitmix64_host(uint64_t x) {
   return z ^ (z >> 31);
 }
 
+// levels of the subdomain-face ring
+int64_t ring_depth(adg_flux flux, const adg_options& o, int np) {
+  if (o.delay_mode == ADG_DELAY_RANDOM)
+    return o.random_delay_max + (flux == ADG_FLUX_STD_DELAYED ? 0 : np) + 1;
+  return flux == ADG_FLUX_STD_DELAYED ? 1 : np + 1;
+}
+
 int num_interfaces(int dim, const int* P) {
   int nsub = 1, dirs = 0;
   for (int d = 0; d < dim; ++d) {
@@ -857,6 +864,13 @@ adg_status adg_create(const adg_mesh* mesh, int degree, const int P[3], int max_
                                       : (int64_t)(degree + 1) * (degree + 1);
     if ((int64_t)(mesh->dim + 2) * ne * nd >= ((int64_t)1 << 31))
       return fail(nullptr, ADG_ERR_UNSUPPORTED, "meshes with 2^31 or more degrees of freedom are not supported");
+    int64_t npe = 0;  // subdomain faces
+    for (int d = 0; d < mesh->dim; ++d)
+      if (P[d] > 1) npe += ne / mesh->n_elem[d] * P[d];
+    if (flux != ADG_FLUX_SYNC &&
+        ring_depth(flux, o, np) * (flux >= ADG_FLUX_AT_TRACE ? 2 : 1) * (mesh->dim + 2) * npe * (nd / (degree + 1)) >=
+            ((int64_t)1 << 31))
+      return fail(nullptr, ADG_ERR_UNSUPPORTED, "delay rings of 2^31 or more values are not supported");
   }
   if (!kernels_available((int)o.precision, mesh->dim, degree + 1))
     return fail(nullptr, ADG_ERR_UNSUPPORTED, "no kernels built for this precision/degree");
@@ -943,10 +957,7 @@ adg_status adg_create(const adg_mesh* mesh, int degree, const int P[3], int max_
       }
       if (s->P[d] > 1) off += nsub;
     }
-    if (o.delay_mode == ADG_DELAY_RANDOM)
-      s->depth = o.random_delay_max + (flux == ADG_FLUX_STD_DELAYED ? 0 : np) + 1;
-    else
-      s->depth = (flux == ADG_FLUX_STD_DELAYED) ? 1 : np + 1;
+    s->depth = (int)ring_depth(flux, o, np);
   }
 
   cudaError_t ce = cudaSuccess;

@@ -15,7 +15,9 @@
 // or one kernel:
 //   vol_faces_kernel(_fp64) : the volume kernel with each element evaluating the numerical flux
 //                 on its own faces from the stored traces (no face-flux array).
-// Index arithmetic is 32-bit: the host rejects meshes with 2^31 or more degrees of freedom.
+// Node and ring indices are 32-bit: the host rejects meshes with 2^31 or more degrees of freedom and
+// rings of 2^31 or more values.  The traces (2 D / N values per degree of freedom) and the face fluxes
+// (D / N) may be larger: their offsets are 64-bit (TraceLay).
 #pragma once
 #include <type_traits>
 #include <cuda_runtime.h>
@@ -310,18 +312,21 @@ template <int D, int N, typename R>
 struct TraceLay {
   static constexpr int NF = IPow<N, D - 1>::value, NV = D + 2;
   static constexpr bool kTogether = std::is_same<R, float>::value;
-  // ds = 2 d + side (side 1: the element's +d face)
-  __device__ static __forceinline__ int at(int ne, int ds, int v, int e, int j) {
-    return kTogether ? ((ds * ne + e) * NF + j) * NV + v : ((ds * NV + v) * ne + e) * NF + j;
+  // ds = 2 d + side (side 1: the element's +d face).  64 bits from the last product on: 2 D NV ne and
+  // 2 D ne NF are at most NV ne ND < 2^31.  (Us per volume launch with the other one of
+  // the last two forms: pairs 48^3 p=3 824 for 745, 32^3 p=5 918 for 867; FP64 48^3 772 for 763.)
+  __device__ static __forceinline__ int64_t at(int ne, int ds, int v, int e, int j) {
+    if (kTogether) return (int64_t)((ds * ne + e) * NF + j) * NV + v;
+    if (std::is_same<R, df64>::value) return (int64_t)(ds * NV + v) * (ne * NF) + (e * NF + j);
+    return (int64_t)((ds * NV + v) * ne + e) * NF + j;
   }
 };
 
 // Layout of the face-flux array: [d][v][e][j], in the FP32 operator [d][e][j][v].
 template <int D, int N, typename R>
 struct FluxLay {
-  static constexpr int NF = IPow<N, D - 1>::value, NV = D + 2;
-  __device__ static __forceinline__ int at(int ne, int d, int v, int e, int j) {
-    return TraceLay<D, N, R>::kTogether ? ((d * ne + e) * NF + j) * NV + v : ((d * NV + v) * ne + e) * NF + j;
+  __device__ static __forceinline__ int64_t at(int ne, int d, int v, int e, int j) {
+    return TraceLay<D, N, R>::at(ne, d, v, e, j);
   }
 };
 
@@ -517,7 +522,7 @@ __device__ __forceinline__ void write_traces_fp64(const MeshArgs& m, const Fixed
 #pragma unroll
     for (int a = 0; a < N; ++a) val[a] = x[a * st];
     line_traces<N>(ft, tab, val, lo, hi);
-    double* dst = tr + ((2 * d * NV + v) * ne + e0) * NF + r;
+    double* dst = tr + TraceLay<D, N, double>::at(ne, 2 * d, v, e0, r);
     dst[0] = lo;
     dst[NV * ne * NF] = hi;
   }
@@ -553,7 +558,7 @@ __device__ __forceinline__ void write_traces(const MeshArgs& m, const OpTables* 
     for (int a = 0; a < N; ++a) t[a] = Arith<C>::tab(tw, twf, a);
     const int el0 = ch * RUN;
     const int el1 = el0 + RUN < EPB ? el0 + RUN : EPB;
-    typename Arith<R>::S* dst = tr + ((ds * NV + v) * ne + e0) * NF + j;
+    typename Arith<R>::S* dst = tr + TraceLay<D, N, R>::at(ne, ds, v, e0, j);
     for (int el = el0; el < el1 && e0 + el < ne; ++el) {
       const C* x = sX + el * SXS + v * ND + base;
       typename Arith<C>::Acc acc = acc_zero(typename Arith<C>::Acc());
@@ -1042,8 +1047,8 @@ __device__ __forceinline__ void vol_body(const VolArgs& A, const SweepArg<D, N, 
           fhi = sFace[(((el * D + d) * 2 + 1) * NV + v) * NF + j];
           flo = sFace[(((el * D + d) * 2 + 0) * NV + v) * NF + j];
         } else {
-          fhi = Arith<R>::load(fl + ((d * NV + v) * ne + e) * NF + j);
-          flo = Arith<R>::load(fl + ((d * NV + v) * ne + elo) * NF + j);
+          fhi = Arith<R>::load(fl + FluxLay<D, N, R>::at(ne, d, v, e, j));
+          flo = Arith<R>::load(fl + FluxLay<D, N, R>::at(ne, d, v, elo, j));
         }
         acc[v] = acc_fma(lm, flo, acc[v]);
         acc[v] = acc_fma(-lp, fhi, acc[v]);
@@ -1207,7 +1212,7 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
         const int lo = (ds & 1) ? e : elem_shift(A.m, e, ec, d, -1);
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-          cp_async8(sFace + ((el * 2 * D + ds) * NV + v) * NF + j, fl + ((d * NV + v) * ne + lo) * NF + j);
+          cp_async8(sFace + ((el * 2 * D + ds) * NV + v) * NF + j, fl + FluxLay<D, N, double>::at(ne, d, v, lo, j));
       }
     } else {
       element_face_fluxes<D, N, double, TT>(faces, A.m, e, ec, el, node, active, smem_raw + SM::FACE_OFF);
@@ -1433,6 +1438,7 @@ __device__ __forceinline__ void face_flux(const FluxArgs& A, int d, int slot, in
   const bool traces = (A.flux_kind >= 3);  // AT on traces, and the learned mode
   const int npe = (int)A.npe;
   const int lvl_stride = (traces ? 2 : 1) * NV * npe * NF;
+  auto at = [=](int v) { return (v * npe + slot) * NF + j; };  // of side and variable v in a level
   int kt = A.uniform_delay;
   if (A.random) {
     const int iface = A.pe_iface[slot];
@@ -1445,8 +1451,8 @@ __device__ __forceinline__ void face_flux(const FluxArgs& A, int d, int slot, in
     S* dst = ring + A.head * lvl_stride;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      Arith<R>::store(dst + (v * npe + slot) * NF + j, wm[v]);
-      Arith<R>::store(dst + ((NV + v) * npe + slot) * NF + j, wp[v]);
+      Arith<R>::store(dst + at(v), wm[v]);
+      Arith<R>::store(dst + at(NV + v), wp[v]);
     }
   }
   if (kt == 0 || (A.store && !traces)) {
@@ -1455,7 +1461,7 @@ __device__ __forceinline__ void face_flux(const FluxArgs& A, int d, int slot, in
     if (A.store && !traces && owner) {
       S* dst = ring + A.head * lvl_stride;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Arith<R>::store(dst + (v * npe + slot) * NF + j, fr[v]);
+      for (int v = 0; v < NV; ++v) Arith<R>::store(dst + at(v), fr[v]);
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) f[v] = fr[v];
@@ -1473,8 +1479,8 @@ __device__ __forceinline__ void face_flux(const FluxArgs& A, int d, int slot, in
       const S* src = ring + lvl * lvl_stride;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        am[v] = acc_fma(c, Arith<R>::load(src + (v * npe + slot) * NF + j), am[v]);
-        if (traces) ap[v] = acc_fma(c, Arith<R>::load(src + ((NV + v) * npe + slot) * NF + j), ap[v]);
+        am[v] = acc_fma(c, Arith<R>::load(src + at(v)), am[v]);
+        if (traces) ap[v] = acc_fma(c, Arith<R>::load(src + at(NV + v)), ap[v]);
       }
     }
     if (traces) {

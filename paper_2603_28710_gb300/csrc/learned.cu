@@ -149,12 +149,12 @@ template <int D, int N, typename R>
 __global__ void log_kernel(const typename Arith<R>::S* tr, const int32_t* face_d,
                            const int32_t* face_e, MeshArgs m, int npe, double* out) {
   constexpr int NF = IPow<N, D - 1>::value, NV = D + 2;
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= 2 * NV * npe * NF) return;
-  const int j = g % NF;
-  const int slot = (g / NF) % npe;
-  const int v = (g / (NF * npe)) % NV;
-  const int side = g / (NF * npe * NV);
+  const int rows = npe * NF;
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= (int64_t)rows * (2 * NV)) return;
+  const int sv = (int)(g / rows), row = (int)(g - (int64_t)sv * rows);
+  const int slot = row / NF, j = row - slot * NF;
+  const int side = sv / NV, v = sv - side * NV;
   const int d = face_d[slot], e = face_e[slot];
   int ec[3];
   elem_coords(m, e, ec);
@@ -162,7 +162,7 @@ __global__ void log_kernel(const typename Arith<R>::S* tr, const int32_t* face_d
   const int ne = (int)m.ne;
   // side 0: high-side trace of e (minus state), side 1: low-side trace of its neighbour
   using Lay = TraceLay<D, N, R>;
-  const int idx = side == 0 ? Lay::at(ne, d * 2 + 1, v, e, j) : Lay::at(ne, d * 2, v, eh, j);
+  const int64_t idx = side == 0 ? Lay::at(ne, d * 2 + 1, v, e, j) : Lay::at(ne, d * 2, v, eh, j);
   out[g] = Arith<R>::to_double(Arith<R>::load(tr + idx));
 }
 
