@@ -148,7 +148,7 @@ struct GradSmem {
 
 __global__ void __launch_bounds__(kGradThreads)
 mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
-                const float* __restrict__ target, int n, float inv_n, float* __restrict__ grad,
+                const float* __restrict__ target, unsigned n, float inv_n, float* __restrict__ grad,
                 float* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   GradSmem& S = *reinterpret_cast<GradSmem*>(smem_raw);
@@ -176,10 +176,11 @@ mlp_grad_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x,
   const int m0 = (warp & 3) * 16, i0 = (warp >> 2) * 32;  // dW2 rows (out) and columns (in)
   __syncthreads();
 
-  const int chunks = (n + kSamples - 1) / kSamples;
+  // (sample numbers are unsigned: the last chunk of 2^31 - 1 samples ends beyond them)
+  const int chunks = (int)((n + kSamples - 1) / kSamples);
   for (int c = blockIdx.x; c < chunks; c += gridDim.x) {
     const int row0 = warp * 16 + g, row1 = row0 + 8;  // rows within the chunk
-    const int s0 = c * kSamples + row0, s1 = s0 + 8;
+    const unsigned s0 = (unsigned)c * kSamples + row0, s1 = s0 + 8;
     float x0[4], x1[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -415,7 +416,7 @@ constexpr int kInferBlocks = 7;  // per SM (72 registers; at 8 it spills, 9 are 
 // conflicts, 72 % of the time in shared-memory wavefronts).  Padded rows and ldmatrix, two
 // column blocks each: 1.97 M samples 456 -> 239 us, 65536 25 -> 15.5 us, the same bits.
 __global__ void __launch_bounds__(32 * kInferWarps, kInferBlocks)
-mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x, int n,
+mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict__ x, unsigned n,
                        float* __restrict__ y) {
   __shared__ __align__(16) float Wf[kW2];               // W1 | b1 (FP32)
   __shared__ __align__(16) float Wo[kMlpParams - kB2];  // b2 | w3 | b3 (FP32)
@@ -428,10 +429,10 @@ mlp_forward_mma_kernel(const uint16_t* __restrict__ pbf, const float* __restrict
   // B fragments of two 8-column blocks per ldmatrix: tile m = lane / 8 holds the rows (outputs)
   // of block m / 2 and the inputs 8 (m % 2) to 8 (m % 2) + 7 of the k-step
   const uint16_t* w2row = &W2[(lane >> 4) * 8 + (lane & 7)][((lane >> 3) & 1) * 8];
-  const int tiles = (n + 15) / 16;
+  const int tiles = (int)((n + 15) / 16);  // (sample numbers unsigned, as in mlp_grad_kernel)
   for (int tile = blockIdx.x * kInferWarps + (threadIdx.x >> 5); tile < tiles;
        tile += gridDim.x * kInferWarps) {
-    const int r0 = tile * 16 + g, r1 = r0 + 8;
+    const unsigned r0 = (unsigned)tile * 16 + g, r1 = r0 + 8;
     float x0[4], x1[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -517,7 +518,7 @@ cudaError_t mlp_infer(const uint16_t* params, const float* x, int64_t n, float* 
   const int64_t tiles = (n + 15) / 16;
   const int64_t want = (tiles + kInferWarps - 1) / kInferWarps;
   const int blocks = (int)(want < 152 * kInferBlocks ? want : 152 * kInferBlocks);
-  mlp_forward_mma_kernel<<<blocks, 32 * kInferWarps, 0, s>>>(params, x, (int)n, y);
+  mlp_forward_mma_kernel<<<blocks, 32 * kInferWarps, 0, s>>>(params, x, (unsigned)n, y);
   return cudaGetLastError();
 }
 
@@ -552,7 +553,7 @@ adg_status adg_mlp_grad(const uint16_t* params_bf16, const float* x, const float
   // blocks of equal numbers of chunks: as few as need the same number of rounds (every block
   // adds its sums to the gradient once, with its rounding)
   const int rounds = (chunks + sms - 1) / sms, grid = (chunks + rounds - 1) / rounds;
-  mlp_grad_kernel<<<grid, kGradThreads, smem, s>>>(params_bf16, x, target, (int)n, 1.0f / (float)n, grad, loss);
+  mlp_grad_kernel<<<grid, kGradThreads, smem, s>>>(params_bf16, x, target, (unsigned)n, 1.0f / (float)n, grad, loss);
   e = cudaGetLastError();
   return e == cudaSuccess ? ADG_OK : mfail(ADG_ERR_CUDA, cudaGetErrorString(e));
 }
