@@ -231,6 +231,20 @@ __global__ void check_finite_kernel(int64_t n, const double* u, int* flag) {
   if (bad) atomicOr(flag, 1);
 }
 
+// FP32 traces of some (d, side) planes between the device's order [ds][row][v] and [ds][v][row] (row =
+// face node of an element).  The copy to or from the host takes longer.
+__global__ void trace_order_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t rows, int NV,
+                                   int planes, bool by_variable) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < planes * rows; i += stride) {
+    const int64_t ds = i / rows, r = i - ds * rows, plane = ds * rows * NV;
+    for (int v = 0; v < NV; ++v) {
+      const int64_t together = plane + r * NV + v, apart = plane + v * rows + r;
+      dst[by_variable ? apart : together] = src[by_variable ? together : apart];
+    }
+  }
+}
+
 VortexParams make_params(const double* lo, const double* h, double gamma, double t, double beta,
                          double x0, double y0, double Lx, double Ly) {
   VortexParams P;
@@ -295,6 +309,12 @@ cudaError_t launch_l2_vortex(int dim, int N, const MeshArgs& m, const double* lo
   for (int d = 0; d < dim; ++d) J *= h[d] / 2.0;
   l2_vortex_kernel<<<nblocks, kRedThreads, 0, s>>>(dim, N, m, P, tab, J, u, partial);
   finish_kernel<false><<<1, kRedThreads, 0, s>>>(3, nblocks, partial, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_trace_order(const float* src, float* dst, int64_t rows, int NV, int planes,
+                               bool by_variable, cudaStream_t s) {
+  trace_order_kernel<<<152 * 16, 256, 0, s>>>(src, dst, rows, NV, planes, by_variable);
   return cudaGetLastError();
 }
 
