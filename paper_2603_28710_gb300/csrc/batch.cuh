@@ -62,17 +62,22 @@ __device__ __forceinline__ void stage_args(T* dst, const T* src) {
 }
 
 // Register budget of the batched volume kernels.  The persistent loop and the arguments
-// read from shared memory raise their register use over the single-instance kernels (FP32:
-// 48 against 32 at 128 threads, over 90 for tiles of 64 threads when left to the
-// compiler), which cuts the occupancy the latency-bound FP32 form needs.  Budgets without
-// spills (ptxas, sm_103a): FP32 40 registers in 2D (48 at N = 4 and 8 and for tiles of at
-// most 64 threads), 56 in 3D; FP64 and FP32 pairs 16 above the single-instance budget
-// (24 at N = 8).
+// read from shared memory raise their register use over the single-instance kernels, which
+// cuts the occupancy that hides their latency; budgets measured best over 48 instances of
+// 20000 (2D) and 30000 nodes each, us per step.  FP64 2D at 48, 56, 64, 72: p=1 1092, 1082, 1076,
+// 1079; p=4 690, 674, 675, 683; p=7 498, 488, 495, 507; 3D at 64, 72, 80, 96: p=1 2895, 2909, 2861,
+// 2858; p=4 3566, 3520, 3472, 3474.  FP32 split 2D at 32, 40, 48, 56: p=2 328, 261, 266, 267; p=4 267,
+// 229, 220, 236; p=7 190, 175, 180, 177; 3D at 40, 48, 56: p=1 698, 761, 762; p=3 564, 606, 621; p=5
+// 310, 252, 251 (a few bytes of spills at these cost less than the occupancy).  Pairs: 16 above the
+// single-instance budget (24 at N = 8).
 template <int D, int N, typename R> struct VolRegs {
   static constexpr int value = VolKernelRegs<D, N, R>::value + (N == 8 ? 24 : 16);
 };
+template <int D, int N> struct VolRegs<D, N, double> {
+  static constexpr int value = D == 2 ? 56 : 80;
+};
 template <int D, int N> struct VolRegs<D, N, float> {
-  static constexpr int value = D != 2 ? 56 : ((N == 4 || N == 8) ? 48 : 40);
+  static constexpr int value = D == 2 ? (N == 5 ? 48 : 40) : (N == 6 ? 48 : 40);
 };
 
 // Sweep table of the instance whose arguments `a` hold, into shared memory (FP32 operator).
@@ -134,7 +139,13 @@ batch_vol_kernel_fp64(const VolArgs* va, int nstages, int stage, BatchGroupArgs 
 // evaluating the numerical fluxes on its own faces, reading each instance's stage and face
 // arguments (the face arguments carry the schedule the device advances) from shared
 // memory.  No face-flux launch.
-template <int D, int N, typename R> struct VolFacesBatchRegs { static constexpr int value = D == 2 ? 72 : 80; };
+// Budget without spills; measured like VolRegs: 2D p=1 at 64 and 72: 345 and 404 us; 3D p=3 at 72 and
+// 80: 752 and 846.  (Smaller ones make equal instances faster still, 2D p=4 246 us at 48 for 277, 3D
+// p=4 1190 for 1531, but the tuner then keeps the large instances of a mixed batch in the graph, where
+// separate handles are faster: 64 instances of 32^2 to 256^2, p=2 to 5, 24.4 for 22.9 ms.)
+template <int D, int N, typename R> struct VolFacesBatchRegs {
+  static constexpr int value = D == 2 ? (N == 2 ? 64 : 72) : (N == 4 ? 72 : 80);
+};
 
 template <int D, int N, typename R, int TT>
 __global__ void __launch_bounds__(vol_block<R>(Tile<D, N, TT>::THREADS),
