@@ -65,9 +65,9 @@ __device__ __forceinline__ int2 fixed_limbs(double x, int es) {
   return make_int2((int)__funnelshift_r(v0, v1, 31), (int)(v0 & 0x7FFFFFFFu));
 }
 
-// c + a b: one wide multiply-add.  (Written in C: inline PTX mad.wide takes two instructions,
-// and so does a product whose operands the compiler knows the sign or range of; the limbs are
-// therefore made opaque where they are computed.)
+// c + a b, a 32x32-bit product added to 64 bits.  Written in C, and with operands that the compiler
+// knows nothing about (opaque), as measured, us per volume launch: 48^3 p=3 765, with mad.wide as
+// inline PTX 919, without the barrier behind the limbs of a trace line 790; 256^2 p=4 117, 135, 120.
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return c + (long long)a * b; }
 __device__ __forceinline__ void opaque(int2& f) { asm("" : "+r"(f.x), "+r"(f.y)); }
 
