@@ -308,19 +308,18 @@ def whole_job_value(work_per_rank_per_step, steps, seconds_max, world):
     return world * work_per_rank_per_step * steps / seconds_max / 1e9
 
 
-def default_path(precision, N, nodes):
-    """The kernel path ADG_PATH_AUTO takes on large meshes: split, except for FP32 with four
-    nodes per direction or fewer than 2^20 nodes (element)."""
-    return "element" if precision == "fp32" and (N == 4 or nodes < 2 ** 20) else "split"
+def path_of(prof):
+    """The kernel path a handle took, from its profile: the element path launches no fluxes."""
+    return "split" if prof["flux"][1] > 0 else "element"
 
 
-def other_path(precision, N, nodes):
-    return "split" if default_path(precision, N, nodes) == "element" else "element"
+def other_path(path):
+    return "split" if path == "element" else "element"
 
 
-def vol_kernel_name(precision, D, N, nodes):
-    """The volume/update kernel the default path runs for an arithmetic."""
-    name = "vol_faces_kernel" if default_path(precision, N, nodes) == "element" else "vol_kernel"
+def vol_kernel_name(precision, D, N, path):
+    """The volume/update kernel of a path for an arithmetic."""
+    name = "vol_faces_kernel" if path == "element" else "vol_kernel"
     return f"{name}{'_fp64' if precision == 'fp64' else ''}<{D},{N}>"
 
 
@@ -383,8 +382,8 @@ def variant_run(adg, stream, precision, steps_per, k, warm, dt, flux="at", delay
     prof = s.get_profile()
     s.set_profiling(False)
     ndof = 4 * N_ELEM * N_ELEM * (DEGREE + 1) ** 2
-    if kernel_path == "auto":  # the path the library chose (only the split path launches fluxes)
-        kernel_path = "split" if prof["flux"][1] > 0 else "element"
+    if kernel_path == "auto":
+        kernel_path = path_of(prof)
     info = s.info()
     finite = s.check_finite()
     err = s.l2_error_vortex(info["t"]) if finite else None  # after warm + k + 2 bench steps
@@ -574,9 +573,9 @@ def tgv_run(adg, stream, mpk, flush, k=3, total_steps=100, with_cpu=True):
         out[prec] = {"value": work * k / (ms * 1e-3) / 1e9,
                      "vol_ms_per_launch": vol_ms / max(vol_n, 1),
                      "flux_ms_per_launch": prof["flux"][0] / max(prof["flux"][1], 1),
-                     "kernel_path": "element" if prof["flux"][1] == 0 else "split",
+                     "kernel_path": path_of(prof),
                      "roofline": dict(roofline_line(prec, 3, TGV_DEGREE + 1, ndof, vol_ms, vol_n,
-                                                    mpk, vol_kernel_name(prec, 3, TGV_DEGREE + 1, ndof // 5)),
+                                                    mpk, vol_kernel_name(prec, 3, TGV_DEGREE + 1, path_of(prof))),
                                       traffic=ncu_traffic(prec, "kernels_3d_traffic"),
                                       traffic_note="ncu capture at 48^3 scaled to 64^3 by the "
                                                    "element count"),
@@ -612,7 +611,7 @@ def tgv_run(adg, stream, mpk, flush, k=3, total_steps=100, with_cpu=True):
     out["fused_path"], out["other_path"] = {}, {}
     for key, prec, path in (("fused_path", "fp64", "fused"), ("fused_path", "df64", "fused"),
                             ("fused_path", "fp32", "fused"),
-                            *(("other_path", p, other_path(p, TGV_DEGREE + 1, ndof // 5))
+                            *(("other_path", p, other_path(out[p]["kernel_path"]))
                               for p in ("fp64", "df64", "fp32"))):
         s = adg.Solver(dim=3, n_elem=(TGV_N,) * 3, degree=TGV_DEGREE, lo=(0, 0, 0),
                        hi=(2 * np.pi,) * 3, P=(TGV_P,) * 3, max_delay=TGV_L, flux="at", rk="ck45",
@@ -792,7 +791,7 @@ def run_gpu(args, rank, world, local_rank):
     vol_ms, vol_n = prof["vol"]
     flux_ms, flux_n = prof["flux"]
     roof = roofline_line(args.precision, 2, DEGREE + 1, ndof, vol_ms, vol_n, mpk,
-                         vol_kernel_name(args.precision, 2, DEGREE + 1, ndof // 4))
+                         vol_kernel_name(args.precision, 2, DEGREE + 1, path_of(prof)))
     roof["traffic"] = ncu_traffic(args.precision)
     launches_per_step = (vol_n + flux_n) / max(args.profile_steps, 1)
 
@@ -832,7 +831,7 @@ def run_gpu(args, rank, world, local_rank):
             prec: {k: v for k, v in variant_run(adg, stream, prec, steps_per, 3, 1, dt,
                                                 kernel_path=path).items()
                    if k in ("value", "vol_ms_per_launch", "flux_ms_per_launch", "kernel_path")}
-            for prec, path in ((p, other_path(p, DEGREE + 1, ndof // 4)) for p in ("fp64", "df64", "fp32"))}
+            for prec, path in ((p, other_path(variants[p]["kernel_path"])) for p in ("fp64", "df64", "fp32"))}
 
     batched = None
     if world == 1 and not args.no_batch:

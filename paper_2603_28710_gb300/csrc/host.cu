@@ -235,13 +235,16 @@ void build_tables(adg_solver* s) {
   long double lp[16], lm[16];
   lagrange_at(N, x, lam, 1.0L, lp);
   lagrange_at(N, x, lam, -1.0L, lm);
-  for (int d = 0; d < 3; ++d) {
+  const int M = N + 2;
+  long double rows[3][kMaxN * (kMaxN + 2)];  // per direction and row N flux weights, low and high face
+  for (int d = 0; d < s->dim; ++d) {
     long double sc = 2.0L / (long double)s->h[d];
     for (int i = 0; i < N; ++i) {
       for (int a = 0; a < N; ++a) {
         long double q = sc * (long double)wd[a] * Dm[a][i] / (long double)wd[i];
         T.Q[d][i * N + a] = (double)q;
         T.Qf[d][i * N + a] = split2(q);
+        rows[d][i * M + a] = q;
       }
       // lift coefficients (2/h) l_i(+-1) / omega_i, halved: the face-flux kernel stores
       // twice the numerical flux
@@ -251,6 +254,8 @@ void build_tables(adg_solver* s) {
       T.Lm[d][i] = (double)vm;
       T.Lpf[d][i] = split2(vp);
       T.Lmf[d][i] = split2(vm);
+      rows[d][i * M + N] = vm;
+      rows[d][i * M + N + 1] = -vp;
     }
   }
   for (int a = 0; a < N; ++a) {
@@ -259,25 +264,16 @@ void build_tables(adg_solver* s) {
     T.Tpf[a] = split2(lp[a]);
     T.Tmf[a] = split2(lm[a]);
   }
-  // the same rows in fixed point: per direction N flux weights, low and high face
+  // the same rows in fixed point
   {
-    const int M = N + 2;
-    long double rows[kMaxN * (kMaxN + 2)];
     for (int d = 0; d < s->dim; ++d) {
-      const long double sc = 2.0L / (long double)s->h[d];
-      for (int i = 0; i < N; ++i) {
-        for (int a = 0; a < N; ++a)
-          rows[i * M + a] = sc * (long double)wd[a] * Dm[a][i] / (long double)wd[i];
-        rows[i * M + N] = 0.5L * sc * lm[i] / (long double)wd[i];
-        rows[i * M + N + 1] = -0.5L * sc * lp[i] / (long double)wd[i];
-      }
-      const long double sum = row_sum_max(rows, N, M);
+      const long double sum = row_sum_max(rows[d], N, M);
       if (!std::isfinite(sum)) {
         s->fix_ok = false;
         continue;
       }
       s->fix_s[d] = fixed_shift(sum);
-      for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[i], s->fix_s[d]));
+      for (int i = 0; i < N * M; ++i) s->fix_q[d][i] = (int64_t)llroundl(ldexpl(rows[d][i], s->fix_s[d]));
     }
     fixed_sweep_tables(s, 0.0, false, &T.fx);
     const int st = fixed_shift(std::max(row_sum_max(lm, 1, N), row_sum_max(lp, 1, N)));

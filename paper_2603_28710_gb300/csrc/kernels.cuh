@@ -292,8 +292,9 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
 constexpr long long kWaitLimitCycles = 2000000000ll;
 
 // Arithmetic of the trace interpolation for an operator arithmetic R: the FP32-pair kernels
-// interpolate in native FP64 (their FP64 pipe is otherwise idle and the RK update hands
-// over the FP64 stage input), the others in R itself.
+// interpolate in native FP64 (the RK update hands over the FP64 stage input), the others in R
+// itself.  These chains are about half of the pair kernels' FP64 operations, whose pipe is 78 % busy
+// (256^2 p=4); in fixed point they cost 15 % more time, as the kernels are bound by issue as well.
 template <typename R> struct TraceCompute { using C = R; };
 template <> struct TraceCompute<df64> { using C = double; };
 
