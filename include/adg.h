@@ -190,7 +190,9 @@ adg_status adg_conservation(adg_solver* s, double* sums);
 adg_status adg_l2_error_vortex(adg_solver* s, double t, double beta, double x0, double y0,
                                double* err3);
 
-/* ADG_OK if every state value is finite, ADG_ERR_NONFINITE otherwise. */
+/* ADG_OK if every state value is finite, ADG_ERR_NONFINITE otherwise.  FP32 and FP32 pairs: finite in
+ * the operator's arithmetic, of magnitude up to 2^127 (a NaN or Inf of the operator enters the FP64
+ * state as a value beyond it). */
 adg_status adg_check_finite(adg_solver* s);
 
 /* ---- checkpoint / resume ---------------------------------------------------------- */

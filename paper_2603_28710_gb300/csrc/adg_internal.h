@@ -252,6 +252,6 @@ cudaError_t launch_l2_vortex(int dim, int N, const MeshArgs& m, const double* lo
                              cudaStream_t s);
 cudaError_t launch_trace_order(const float* src, float* dst, int64_t rows, int NV, int planes,
                                bool by_variable, cudaStream_t s);
-cudaError_t launch_check_finite(int64_t n, const double* u, int* flag, cudaStream_t s);
+cudaError_t launch_check_finite(int64_t n, const double* u, double largest, int* flag, cudaStream_t s);
 
 }  // namespace adg

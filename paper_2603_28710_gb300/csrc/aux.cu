@@ -223,11 +223,11 @@ __global__ void l2_vortex_kernel(int dim, int N, MeshArgs m, VortexParams P, con
   }
 }
 
-__global__ void check_finite_kernel(int64_t n, const double* u, int* flag) {
+__global__ void check_finite_kernel(int64_t n, const double* u, double largest, int* flag) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int bad = 0;
-  for (; i < n; i += stride) bad |= !isfinite(u[i]);
+  for (; i < n; i += stride) bad |= !(fabs(u[i]) <= largest);
   if (bad) atomicOr(flag, 1);
 }
 
@@ -318,9 +318,9 @@ cudaError_t launch_trace_order(const float* src, float* dst, int64_t rows, int N
   return cudaGetLastError();
 }
 
-cudaError_t launch_check_finite(int64_t n, const double* u, int* flag, cudaStream_t s) {
+cudaError_t launch_check_finite(int64_t n, const double* u, double largest, int* flag, cudaStream_t s) {
   cudaMemsetAsync(flag, 0, sizeof(int), s);
-  check_finite_kernel<<<152 * 8, 256, 0, s>>>(n, u, flag);
+  check_finite_kernel<<<152 * 8, 256, 0, s>>>(n, u, largest, flag);
   return cudaGetLastError();
 }
 

@@ -5,7 +5,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <new>
 #include <string>
@@ -1383,7 +1385,10 @@ adg_status adg_l2_error_vortex(adg_solver* s, double t, double beta, double x0, 
 
 adg_status adg_check_finite(adg_solver* s) {
   if (!s) return fail(nullptr, ADG_ERR_INVALID, "handle is NULL");
-  ADG_CUDA(s, launch_check_finite(s->ndof, s->w, s->flag, s->stream));
+  // the FP32 and pair operators add their increments to the FP64 solution through an integer
+  // conversion (arith.cuh) that turns Inf and NaN into finite values of 2^128 and more
+  const double largest = s->prec == 0 ? std::numeric_limits<double>::max() : std::ldexp(1.0, 127);
+  ADG_CUDA(s, launch_check_finite(s->ndof, s->w, largest, s->flag, s->stream));
   int f = 0;
   ADG_CUDA(s, cudaMemcpyAsync(&f, s->flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
   ADG_CUDA(s, cudaStreamSynchronize(s->stream));

@@ -1,5 +1,6 @@
 """A time step that is not finite is visible in the FP64 operator's state: also of a uniform gas,
-whose right-hand side is rounding noise, a step with it leaves no variable finite at any node.
+whose right-hand side is rounding noise, a step with it leaves no variable finite at any node.  In
+FP32 and FP32 pairs adg_check_finite reports it.
 """
 import numpy as np
 import pytest
@@ -44,3 +45,16 @@ def test_infinite_time_step_in_a_batch():
     b.step(1)
     for i in range(2):
         assert not np.isfinite(b.get_state(i)).any()
+
+
+@pytest.mark.parametrize("path", ["split", "element", "fused"])
+@pytest.mark.parametrize("precision", ["df64", "fp32"])
+@pytest.mark.parametrize("rk", ["ck45", "rk33"])
+@pytest.mark.parametrize("step", [{"dt": np.inf}, {"cfl": np.inf}])
+def test_the_check_sees_it_in_the_other_arithmetics(step, rk, precision, path):
+    s = adg.Solver(n_elem=(6, 5), degree=2, rk=rk, precision=precision, kernel_path=path, **step)
+    s.init_vortex()
+    assert s.check_finite()
+    s.step(1)
+    assert not s.check_finite()
+    s.close()
