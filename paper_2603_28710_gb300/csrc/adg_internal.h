@@ -204,14 +204,17 @@ cudaError_t launch_log_traces(int prec, int dim, int N, const void* tr, const in
                               const int32_t* face_e, const MeshArgs& m, int64_t npe, double* out,
                               cudaStream_t s);
 
-// ADG_PATH_AUTO: whether the element path is the faster one.  FP32 only (the FP64 operator would
-// evaluate every interior face twice on the pipe that bounds it, and so would the pairs).
-// FP32, GB300, us per stage element / split: one launch instead of two up to about 10^6 nodes
-// (35^2 p=4 3.2 / 4.5, 100^2 8.6 / 9.1, 141^2 12.9 / 13.7; 16^3 p=3 13.3 / 13.7); above, the
-// second evaluation of every interior face costs more than the launch and the flux array
-// (256^2 p=4 47.7 / 47.1, 640^2 p=1 60.0 / 56.6, 64^3 p=2 424 / 366, 40^3 p=4 382 / 342, 32^3
-// p=5 329 / 315), except with four nodes per direction, whose tiles fill their warps in every
-// phase (320^2 p=3 42.9 / 45.5, 48^3 289 / 288).
+// ADG_PATH_AUTO: whether the element path is the faster one; GB300, us per stage element / split.
+// FP32: one launch instead of two up to about 10^6 nodes (35^2 p=4 3.8 / 5.4, 100^2 8.5 / 9.6, 141^2
+// 14.2 / 15.3; 20^3 p=1 6.6 / 7.1, 12^3 p=4 11.2 / 12.2); above, the second evaluation of every
+// interior face costs more than the launch and the flux array (256^2 p=4 48.0 / 45.6, 640^2 p=1
+// 59.9 / 55.7, 64^3 p=2 399 / 358, 40^3 p=4 349 / 332, 32^3 p=5 328 / 307), except with four nodes
+// per direction, whose tiles fill their warps in every phase (200^2 p=3 16.5 / 17.8, 320^2 42.7 /
+// 45.3, 1024^2 378 / 416, 96^3 2162 / 2203; but 24^3 43.2 / 39.7, 48^3 290 / 285).  FP64 and pairs
+// would evaluate every interior face twice on the pipe that bounds them, or in the latency that
+// bounds small meshes: FP64 16^2 p=2 12.7 / 10.4, 64^2 16.5 / 12.8, 256^2 p=4 241 / 177, 8^3 p=3 15.2 /
+// 13.4; pairs 10.1 / 9.7, 11.1 / 11.0, 173 / 131, 12.5 / 13.1 (only 16^2 p=4 gains more: FP64 9.5 / 10.6,
+// pairs 8.7 / 10.1).
 inline bool element_path_faster(int prec, int N, int64_t nodes) {
   return prec == 1 && (N == 4 || nodes < ((int64_t)1 << 20));
 }
