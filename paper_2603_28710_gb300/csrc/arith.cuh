@@ -109,7 +109,7 @@ __device__ __forceinline__ float r_sqrt(float x) {
 // iteration; both to about 2^-43), then the correction g + (m - g^2) / (2 sqrt(m)) with the exact
 // residual (error 2^-86 before the last rounding): 6 FP64 operations instead of the IEEE
 // sequence's about 20.  (Without the step for 1/(2 sqrt(m)), 5 operations: 2^-13 of the results
-// rounded the other way; a binomial series in 5: errors up to 0.8 ulp.)  Zero, subnormal,
+// rounded the other way; a binomial series in 5: errors up to 0.75 ulp.)  Zero, subnormal,
 // negative and non-finite arguments take sqrt().
 __device__ __forceinline__ double half_sqrt(double s) {
   const int hi = __double2hiint(s);

@@ -150,8 +150,11 @@ __device__ __forceinline__ C interp_line(const C (&t)[N], const C* x, int stride
   return acc_result(acc);
 }
 
-// Register budget of the fused kernel (no spills, ptxas sm_103a).
+// Register budget of the fused kernel (FP32 without spills; the others spill up to 250 bytes, which
+// costs less than the occupancy).  FP64, us per stage at 56, 64, 80: 256^2 p=4 324, 331, 353; 216^2 p=5
+// 311, 296, 339; 48^3 p=3 3151, 3151, 2996; 40^3 p=4 4317, 4316, 4078.
 template <int D, int N, typename R> struct FusedRegs { static constexpr int value = 64; };
+template <int D, int N> struct FusedRegs<D, N, double> { static constexpr int value = D == 2 ? 64 : 80; };
 template <int D, int N> struct FusedRegs<D, N, float> { static constexpr int value = D == 2 ? 56 : 64; };
 
 template <int D, int N, typename R>

@@ -1375,7 +1375,7 @@ __device__ __forceinline__ void vol_body_fp64(const VolArgs& A, int tile, unsign
 // compiler from trading occupancy for registers).  The FP32 form is latency-bound and
 // wants every warp slot.
 template <int D, int N, typename R> struct VolKernelRegs {
-  static constexpr int value = (D == 2 && (N == 2 || N == 8)) ? 64 : 56;  // no spills (ptxas)
+  static constexpr int value = (D == 2 && (N == 2 || N == 8)) ? 64 : 56;  // at most 4 bytes spill (ptxas)
 };
 template <int D, int N> struct VolKernelRegs<D, N, double> {
   // us at 48, 56, 64 registers: 256^2 p=4 118.0, 117.3, 118.4; 640^2 p=1 151, 143, 141; 160^2 p=7
@@ -1562,8 +1562,8 @@ __device__ __forceinline__ void element_face_fluxes(const ElementFaces& F, const
 
 // One launch per RK stage without the face-flux launch: the volume kernel with every
 // element evaluating the numerical fluxes on its own faces (ElementFaces).  Register
-// budgets: no spills (ptxas sm_103a); the FP32 form measured best at 48 over the degrees (40:
-// up to 30 % slower, 56: 1 to 5 %).
+// budgets: no spills (ptxas sm_103a; FP64 3D p=5: 16 bytes); the FP32 form measured best at 48
+// over the degrees (40: up to 30 % slower, 56: 1 to 5 %).
 template <int D, int N, typename R> struct VolFacesRegs { static constexpr int value = D == 2 ? 64 : 80; };
 template <int D, int N> struct VolFacesRegs<D, N, float> { static constexpr int value = 48; };
 template <int D, int N> struct VolFacesRegs<D, N, double> { static constexpr int value = D == 2 ? 72 : 80; };
